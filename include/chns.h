@@ -166,11 +166,11 @@ void chns_mesh_destroy(chns_mesh* mesh);
  *   CHNS_APPLY_PATCH:  one CTA per patch (a run of <= 256 Morton-consecutive elements whose
  *                      nodes are gathered once into shared memory).
  *   CHNS_APPLY_STREAM: persistent CTAs, each walking the patches blockIdx, blockIdx + grid, ...
- *                      and gathering the next patch's node values into shared memory (cp.async)
- *                      while the current patch is computed. Used by the FP32 Poisson and mass
- *                      applies (including the apply fused into CG); the other operators and
- *                      precisions keep CHNS_APPLY_PATCH.
- *   CHNS_APPLY_AUTO:   CHNS_APPLY_STREAM when the mesh has at least 16 patches per SM.
+ *                      with two leaves per thread and the next patch's node values loaded while
+ *                      the current patch is computed. Used by the FP32 Poisson and mass applies,
+ *                      with FP32 or bfloat16 coefficients (including the apply fused into CG);
+ *                      the other operators and precisions keep CHNS_APPLY_PATCH.
+ *   CHNS_APPLY_AUTO:   CHNS_APPLY_STREAM when the mesh has at least 8 patches per SM.
  * max_ctas bounds the persistent grid (0: as many CTAs as the device holds at once). Errors:
  * EINVAL for a null mesh, an unknown kernel or max_ctas < 0. Not thread-safe against applies
  * running on the same mesh from other host threads. */

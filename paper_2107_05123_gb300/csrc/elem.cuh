@@ -24,6 +24,7 @@ constexpr double kW1 = 0.21132486540518711775;  // (1 - 1/sqrt(3)) / 2
 template <class T>
 struct PrmT {
   T alpha, beta, gamma, xi, C_I;
+  T rho_m, eta_m;                       // rho_-, eta_- (phi = -1)
   T dt, idt, four_idt2, k2dt, half_dt;  // dt, 1/dt, 4/dt^2, 2/dt, dt/2
   T inv_re, h2re, inv_pe, h2pe;         // 1/Re, 1/(2Re), 1/Pe, 1/(2Pe)
   T inv_pecn, kmu, kphi, cn2;           // 1/(Pe Cn), 1/(2 Pe Cn), Cn^2/2, Cn^2
@@ -56,6 +57,8 @@ inline PrmT<T> make_prm(const chns_params& p) {
   q.gamma = (T)gamma;
   q.xi = (T)xi;
   q.C_I = (T)p.C_I;
+  q.rho_m = (T)rm;
+  q.eta_m = (T)em;
   q.dt = (T)p.dt;
   q.idt = (T)(1.0 / p.dt);
   q.four_idt2 = (T)(4.0 / (p.dt * p.dt));

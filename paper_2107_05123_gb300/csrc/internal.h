@@ -27,9 +27,18 @@ constexpr int kPatchSlots = 640;
 constexpr uint32_t kElocSlotMask = 0x3ff;
 constexpr int kElocLevelShift = 10;
 constexpr uint32_t kElocLevelMask = 0x1f;
-// The persistent, pipelined apply is chosen automatically once the mesh has at least this many
-// patches per SM.
-constexpr int kStreamMinPatchesPerSm = 16;
+// FP32 applies take two leaves of a patch per thread: brick pairs (a brick is the 8 children of
+// one octant, all of them leaves; its four pairs are x-neighbours) come first, then the other
+// leaves two by two.
+constexpr int kTileThreads = 128;
+static_assert(2 * kTileThreads == kPatchElems && 4 * kPatchSlots <= 0x1000, "references");
+// Head of a patch: first 16-byte unit of its index record; regular | hanging slots << 16; bricks |
+// other leaves << 16; lowest level | units from the record to its references << 16. Sections of
+// the record (32-bit words, each on a 16-byte boundary):
+//   regular slots: node id | kOwnBit | kDirBit, ascending node ids;
+//   parents: per hanging slot four local slots (two parents: a, b, a, b);
+//   references of the brick pairs, [3][pairs] x 8 bytes, and of the others, [2][pairs] x 16 bytes:
+//     12 or 16 entries of 16 bits (see PairRefs).
 
 // Element geometry of one octant level on the box [0,L]^3 scaled per axis: h_d = L_d 2^-level,
 // 1/h_d and det J = h_x h_y h_z / 8, in FP64 and FP32 (looked up, never recomputed per element).
@@ -51,10 +60,8 @@ struct MeshDev {
   // patch tables
   int64_t n_patch;
   const int32_t* patch_elem;  // [n_patch+1] first element of each patch
-  const int32_t* patch_slot;  // [n_patch+1] first slot of each patch (regular slots, then hanging)
-  const int32_t* patch_nreg;  // [n_patch] regular slots of each patch
-  const int32_t* slot_node;   // [slots] regular slot: node id | kOwnBit | kDirBit
-  const ushort4* slot_par;    // [slots] hanging slot: local parent slots (0xffff = none)
+  const uint4* patch_head;    // [n_patch] heads
+  const uint32_t* rec;        // index records
   const uint4* eloc;          // [n_elem] 8 local slot indices (uint16) per element + level
   const LevelGeo* geo;        // [CHNS_MAXD] per-level geometry
 };
@@ -93,14 +100,11 @@ struct chns_mesh {
   uint32_t* d_anchor = nullptr;
   int32_t* d_bnd = nullptr;          // boundary node indices (n_boundary)
   int32_t* d_patch_elem = nullptr;
-  int32_t* d_patch_slot = nullptr;
-  int32_t* d_patch_nreg = nullptr;
-  int32_t* d_slot_node = nullptr;
-  ushort4* d_slot_par = nullptr;
+  uint4* d_patch_head = nullptr;
+  uint32_t* d_rec = nullptr;
   uint4* d_eloc = nullptr;
   chns::LevelGeo* d_geo = nullptr;
   uint32_t* d_node_int = nullptr;    // node coordinates (3*n_nodes, units 2^-CHNS_MAXD)
-  int64_t n_slots = 0;
   chns::Workspace ws;
   cudaStream_t cap_stream = nullptr;  // private stream used only to capture CUDA graphs
   // quadrature data of the momentum operator during a momentum solve (see momentum_qdata_on)

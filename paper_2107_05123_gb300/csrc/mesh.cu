@@ -14,6 +14,7 @@
 #include <atomic>
 #include <cmath>
 #include <cstring>
+#include <memory>
 #include <numeric>
 #include <thread>
 
@@ -120,10 +121,8 @@ void free_mesh(chns_mesh* m) {
   dfree(m->d_anchor);
   dfree(m->d_bnd);
   dfree(m->d_patch_elem);
-  dfree(m->d_patch_slot);
-  dfree(m->d_patch_nreg);
-  dfree(m->d_slot_node);
-  dfree(m->d_slot_par);
+  dfree(m->d_patch_head);
+  dfree(m->d_rec);
   dfree(m->d_eloc);
   dfree(m->d_geo);
   dfree(m->d_node_int);
@@ -149,12 +148,15 @@ void free_mesh(chns_mesh* m) {
   delete m;
 }
 
-// Greedy partition of the Morton-ordered elements into patches (see kPatchElems/kPatchSlots):
-// regular slots = distinct nodes used as corners or as parents of hanging corners, hanging slots
-// = distinct hanging corners; a node is owned by a patch when no other patch has it as a slot.
+// Greedy partition of the Morton-ordered elements into patches (see kPatchElems/kPatchSlots and
+// the index record in internal.h): regular slots = distinct nodes used as corners or as parents
+// of hanging corners, hanging slots = distinct hanging corners; a node is owned by a patch when no
+// other patch has it as a slot. Bricks are never split. The leaf list is cut into chunks of
+// kPatchChunk leaves (moved to the next unit) that are partitioned in parallel.
 struct PatchTables {
-  std::vector<int32_t> elem, slot, nreg, node;
-  std::vector<ushort4> par;
+  std::vector<int32_t> elem;  // per patch: first element
+  std::vector<uint4> head;
+  std::vector<uint32_t> rec;
   std::vector<uint4> eloc;
 };
 
@@ -162,109 +164,275 @@ static_assert(kPatchSlots - 1 <= (int)kElocSlotMask && CHNS_MAXD - 1 <= (int)kEl
                   kElocLevelShift + 5 <= 16,
               "patch slot and level must fit the first uint16 of eloc");
 
-static void build_patches(int64_t n, int64_t N, const std::vector<int32_t>& enode,
-                          const std::vector<int4>& hang, const uint8_t* levels, PatchTables& P) {
-  std::vector<int32_t> stamp_n(N, -1), slot_n(N, 0), stamp_h(hang.size(), -1), slot_h(hang.size(), 0);
-  std::vector<int32_t> count(N, 0);
-  std::vector<int32_t> reg, hg;                    // current patch: node ids, hanging ids
-  std::vector<std::array<int32_t, 8>> ecorner;     // provisional: >= 0 regular slot, < 0 ~hslot
-  int32_t pid = 0;
-  int64_t e0 = 0;
-  P.eloc.resize(n);
-  auto close = [&](int64_t e_end) {
-    const int32_t nr = (int32_t)reg.size();
-    P.elem.push_back((int32_t)e0);
-    P.slot.push_back((int32_t)P.node.size());
-    P.nreg.push_back(nr);
-    for (int32_t id : reg) {
-      P.node.push_back(id);
-      P.par.push_back(make_ushort4(0xffff, 0xffff, 0xffff, 0xffff));
-      ++count[id & kIdxMask & ~kDirBit];
+constexpr int64_t kPatchChunk = 32768;
+
+namespace {
+
+// Distinct keys of one patch with the slot each gets (open addressing, cleared by epoch).
+class SlotMap {
+ public:
+  SlotMap() : key_(kSize), val_(kSize), epoch_(kSize, 0) {}
+  void clear() { ++now_; }
+  // position of the key; *fresh: it was not there
+  int put(uint32_t k, bool* fresh) {
+    uint32_t h = (k * 2654435761u) >> (32 - kBits);
+    while (epoch_[h] == now_ && key_[h] != k) h = (h + 1) & (kSize - 1);
+    *fresh = epoch_[h] != now_;
+    if (*fresh) {
+      epoch_[h] = now_;
+      key_[h] = k;
     }
-    for (int32_t h : hg) {
-      const int4 q = hang[h];
-      const int32_t ps[4] = {q.x, q.y, q.z, q.w};
-      unsigned short loc[4] = {0xffff, 0xffff, 0xffff, 0xffff};
-      for (int k = 0; k < 4; ++k)
-        if (ps[k] >= 0) loc[k] = (unsigned short)slot_n[ps[k] & kIdxMask];
-      P.node.push_back(-1);
-      P.par.push_back(make_ushort4(loc[0], loc[1], loc[2], loc[3]));
-    }
-    for (int64_t e = e0; e < e_end; ++e) {
-      unsigned short l[8];
-      for (int c = 0; c < 8; ++c) {
-        int32_t v = ecorner[e - e0][c];
-        l[c] = (unsigned short)(v >= 0 ? v : nr + ~v);
+    return (int)h;
+  }
+  void erase_last(int pos) { epoch_[pos] = 0; }  // of the latest insertions, newest first
+  int32_t& val(int pos) { return val_[pos]; }
+  int32_t get(uint32_t k) {
+    uint32_t h = (k * 2654435761u) >> (32 - kBits);
+    while (epoch_[h] != now_ || key_[h] != k) h = (h + 1) & (kSize - 1);
+    return val_[h];
+  }
+
+ private:
+  static constexpr int kBits = 12, kSize = 1 << kBits;
+  std::vector<uint32_t> key_;
+  std::vector<int32_t> val_;
+  std::vector<uint32_t> epoch_;
+  uint32_t now_ = 0;
+};
+
+struct PatchBuilder {
+  int64_t N;
+  const std::vector<int32_t>& enode;
+  const std::vector<int4>& hang;
+  const uint8_t* levels;
+  const std::vector<uint8_t>& unit;  // per leaf: 8 at the first leaf of a brick, else 1
+  std::vector<uint4>& eloc;
+  std::vector<int32_t> elem;
+  std::vector<uint4> head;
+  std::vector<uint32_t> rec;
+
+  SlotMap map;
+  std::vector<int32_t> reg, hg;  // ids of the current patch (node id with flags; hanging id)
+  std::vector<int> fresh;
+
+  int32_t slot_of(int32_t v) { return map.get((uint32_t)(v & kIdxMask)); }
+
+  // adds the nodes of one unit; returns false (and takes them back) if the slots do not fit
+  bool add_unit(int64_t e, int n, bool force) {
+    const size_t r0 = reg.size(), h0 = hg.size();
+    fresh.clear();
+    auto node = [&](int32_t id) {
+      bool f;
+      const int pos = map.put((uint32_t)(id & kIdxMask), &f);
+      if (f) {
+        fresh.push_back(pos);
+        reg.push_back(id);
       }
-      l[0] = (unsigned short)(l[0] | ((uint32_t)levels[e] << kElocLevelShift));
-      P.eloc[e] = make_uint4(l[0] | (l[1] << 16), l[2] | (l[3] << 16), l[4] | (l[5] << 16),
-                             l[6] | (l[7] << 16));
+    };
+    for (int64_t q = 8 * e; q < 8 * (e + n); ++q) {
+      const int32_t v = enode[q], j = v & kIdxMask;
+      if (j < N) {
+        node(v);
+        continue;
+      }
+      bool f;
+      const int pos = map.put((uint32_t)j, &f);
+      if (!f) continue;
+      fresh.push_back(pos);
+      const int32_t h = j - (int32_t)N;
+      hg.push_back(h);
+      const int4 p = hang[h];
+      node(p.x);
+      node(p.y);
+      if (p.z >= 0) {
+        node(p.z);
+        node(p.w);
+      }
     }
+    if (force || reg.size() + hg.size() <= (size_t)kPatchSlots) return true;
+    while (!fresh.empty()) {
+      map.erase_last(fresh.back());
+      fresh.pop_back();
+    }
+    reg.resize(r0);
+    hg.resize(h0);
+    return false;
+  }
+
+  void close(int64_t e0, int64_t e1, const std::vector<std::pair<int32_t, int32_t>>& units) {
+    std::sort(reg.begin(), reg.end(),
+              [](int32_t a, int32_t b) { return (a & kIdxMask) < (b & kIdxMask); });
+    std::sort(hg.begin(), hg.end());
+    const int nr = (int)reg.size(), nh = (int)hg.size();
+    bool f;
+    for (int i = 0; i < nr; ++i) map.val(map.put((uint32_t)(reg[i] & kIdxMask), &f)) = i;
+    for (int i = 0; i < nh; ++i) map.val(map.put((uint32_t)(N + hg[i]), &f)) = nr + i;
+    // corner slots of the elements
+    std::vector<std::array<uint16_t, 8>> loc((size_t)(e1 - e0));
+    for (int64_t e = e0; e < e1; ++e) {
+      auto& l = loc[e - e0];
+      for (int c = 0; c < 8; ++c) l[c] = (uint16_t)slot_of(enode[8 * e + c]);
+      eloc[e] = make_uint4((l[0] | (uint32_t)levels[e] << kElocLevelShift) | (uint32_t)l[1] << 16,
+                           l[2] | (uint32_t)l[3] << 16, l[4] | (uint32_t)l[5] << 16,
+                           l[6] | (uint32_t)l[7] << 16);
+    }
+    std::vector<uint32_t> w;
+    auto align = [&] { w.resize((w.size() + 3) / 4 * 4, 0); };
+    for (int32_t id : reg) w.push_back((uint32_t)id);
+    align();
+    for (int i = 0; i < nh; ++i) {
+      const int4 q = hang[hg[i]];
+      const uint32_t ab = (uint32_t)slot_of(q.x) | (uint32_t)slot_of(q.y) << 16;
+      w.push_back(ab);
+      w.push_back(q.z < 0 ? ab : (uint32_t)slot_of(q.z) | (uint32_t)slot_of(q.w) << 16);
+    }
+    align();
+    // references: brick pairs, then the other leaves two by two
+    const uint32_t refs = (uint32_t)(w.size() / 4);
+    int nb = 0, ns = 0, low = CHNS_MAXD;
+    for (auto& u : units) {
+      (u.second == 8 ? nb : ns) += 1;
+      low = std::min(low, (int)levels[u.first]);
+    }
+    const int nb4 = 4 * nb, n2 = (ns + 1) / 2;
+    std::vector<std::array<uint16_t, 16>> ref((size_t)(nb4 + n2));
+    // level and number of leaf k of the patch in the upper bits of entries at, at + 2, at + 4
+    auto tag = [&](std::array<uint16_t, 16>& r, int at, int k) {
+      r[at] = (uint16_t)(r[at] | (uint32_t)(levels[e0 + k] - low) << 12);
+      r[at + 2] = (uint16_t)(r[at + 2] | (uint32_t)(k & 15) << 12);
+      r[at + 4] = (uint16_t)(r[at + 4] | (uint32_t)(k >> 4) << 12);
+    };
+    int b = 0, s = 0;
+    for (auto& u : units) {
+      const int k0 = (int)(u.first - e0);
+      if (u.second == 8) {
+        for (int p = 0; p < 4; ++p) {
+          const int lo = k0 + 2 * p;
+          auto& r = ref[4 * b + p];
+          for (int j = 0; j < 4; ++j)
+            for (int ix = 0; ix < 3; ++ix)
+              r[3 * j + ix] = (uint16_t)(4 * (ix < 2 ? loc[lo][ix + 2 * j] : loc[lo + 1][1 + 2 * j]));
+          tag(r, 0, lo);
+        }
+        ++b;
+      } else {
+        auto& r = ref[nb4 + s / 2];
+        for (int a = 0; a < 8; ++a) {
+          r[8 * (s & 1) + a] = (uint16_t)(4 * loc[k0][a]);
+          if (!(s & 1)) r[8 + a] = r[a];  // until there is a second leaf
+        }
+        tag(r, 8 * (s & 1), k0);
+        if (s & 1) r[6] = (uint16_t)(r[6] | 1u << 12);
+        ++s;
+      }
+    }
+    auto put = [&](const std::array<uint16_t, 16>& r, int from, int halves) {
+      for (int k = from; k < from + halves; k += 2)
+        w.push_back((uint32_t)r[k] | (uint32_t)r[k + 1] << 16);
+    };
+    for (int j = 0; j < 3; ++j)
+      for (int t = 0; t < nb4; ++t) put(ref[t], 4 * j, 4);
+    align();
+    for (int j = 0; j < 2; ++j)
+      for (int t = 0; t < n2; ++t) put(ref[nb4 + t], 8 * j, 8);
+    align();
+    elem.push_back((int32_t)e0);
+    head.push_back(make_uint4((uint32_t)(rec.size() / 4), (uint32_t)nr | (uint32_t)nh << 16,
+                              (uint32_t)nb | (uint32_t)ns << 16, (uint32_t)low | refs << 16));
+    rec.insert(rec.end(), w.begin(), w.end());
     reg.clear();
     hg.clear();
-    ecorner.clear();
-    ++pid;
-    e0 = e_end;
+    map.clear();
+  }
+
+  void run(int64_t b, int64_t e) {
+    std::vector<std::pair<int32_t, int32_t>> units;
+    map.clear();
+    int64_t e0 = b;
+    for (int64_t i = b; i < e;) {
+      const int n = unit[i];
+      if (i - e0 + n > kPatchElems || !add_unit(i, n, i == e0)) {
+        close(e0, i, units);
+        units.clear();
+        e0 = i;
+        continue;
+      }
+      units.push_back({(int32_t)i, n});
+      i += n;
+    }
+    if (e0 < e) close(e0, e, units);
+  }
+};
+
+}  // namespace
+
+static void build_patches(int64_t n, int64_t N, const uint32_t* anchors,
+                          const std::vector<int32_t>& enode, const std::vector<int4>& hang,
+                          const uint8_t* levels, PatchTables& P) {
+  // bricks: 8 consecutive leaves of one level, the first at its parent's anchor
+  std::vector<uint8_t> unit((size_t)n, 1);
+  for (int64_t e = 0; e + 8 <= n;) {
+    const int l = levels[e];
+    bool brick = l > 0;
+    const uint32_t sp = l > 0 ? (uint32_t)(kFull >> (l - 1)) : 1;
+    for (int d = 0; d < 3 && brick; ++d) brick = anchors[3 * e + d] % sp == 0;
+    for (int k = 1; k < 8 && brick; ++k) brick = levels[e + k] == l;
+    if (brick) unit[e] = 8;
+    e += brick ? 8 : 1;
+  }
+  std::vector<int64_t> cut{0};
+  for (int64_t c = kPatchChunk; c < n; c += kPatchChunk) {
+    int64_t e = c;  // not inside a brick
+    for (int k = 1; k < 8; ++k)
+      if (unit[c - k] == 8) e = c - k + 8;
+    if (e < n && e > cut.back()) cut.push_back(e);
+  }
+  cut.push_back(n);
+  P.eloc.resize(n);
+  const int nc = (int)cut.size() - 1;
+  std::vector<std::unique_ptr<PatchBuilder>> part(nc);
+  std::atomic<int> next(0);
+  std::atomic<bool> failed(false);
+  auto work = [&] {
+    for (int c; (c = next.fetch_add(1)) < nc;) try {
+        part[c].reset(new PatchBuilder{N, enode, hang, levels, unit, P.eloc});
+        part[c]->run(cut[c], cut[c + 1]);
+      } catch (const std::bad_alloc&) {  // no exception leaves a thread
+        failed.store(true);
+      }
   };
-  for (int64_t e = 0; e < n; ++e) {
-    // distinct new references of this element
-    int32_t newn[40], newh[8];
-    int nn = 0, nh = 0;
-    auto add_node = [&](int32_t id) {
-      const int32_t j = id & kIdxMask;
-      if (stamp_n[j] == pid) return;
-      for (int k = 0; k < nn; ++k)
-        if ((newn[k] & kIdxMask) == j) return;
-      newn[nn++] = id;
-    };
-    for (int c = 0; c < 8; ++c) {
-      const int32_t v = enode[8 * e + c];
-      const int32_t j = v & kIdxMask;
-      if (j < N) {
-        add_node(v);
-      } else {
-        const int32_t h = j - (int32_t)N;
-        bool seen = stamp_h[h] == pid;
-        for (int k = 0; k < nh && !seen; ++k) seen = newh[k] == h;
-        if (!seen) newh[nh++] = h;
-        const int4 q = hang[h];
-        add_node(q.x);
-        add_node(q.y);
-        if (q.z >= 0) {
-          add_node(q.z);
-          add_node(q.w);
-        }
+  const int nt = (int)std::max(1u, std::min(16u, std::thread::hardware_concurrency()));
+  std::vector<std::thread> th;
+  for (int t = 1; t < std::min(nt, nc); ++t) th.emplace_back(work);
+  work();
+  for (auto& t : th) t.join();
+  if (failed.load()) throw std::bad_alloc();
+  // concatenate; a node is owned by the only patch that has it as a regular slot
+  std::vector<uint8_t> count((size_t)N, 0);
+  for (auto& p : part) {
+    const uint32_t base = (uint32_t)(P.rec.size() / 4);
+    for (size_t k = 0; k < p->head.size(); ++k) {
+      uint4 h = p->head[k];
+      const uint32_t* r = &p->rec[4 * (size_t)h.x];
+      h.x += base;
+      P.elem.push_back(p->elem[k]);
+      P.head.push_back(h);
+      for (uint32_t i = 0; i < (h.y & 0xffffu); ++i) {
+        uint8_t& c = count[r[i] & kNodeMask];
+        c = (uint8_t)std::min(2, c + 1);
       }
     }
-    const int64_t slots = (int64_t)reg.size() + hg.size() + nn + nh;
-    if (e > e0 && (e - e0 >= kPatchElems || slots > kPatchSlots)) {
-      close(e);
-      --e;  // re-examine this element in the new patch
-      continue;
-    }
-    for (int k = 0; k < nn; ++k) {
-      const int32_t j = newn[k] & kIdxMask;
-      stamp_n[j] = pid;
-      slot_n[j] = (int32_t)reg.size();
-      reg.push_back(newn[k]);
-    }
-    for (int k = 0; k < nh; ++k) {
-      stamp_h[newh[k]] = pid;
-      slot_h[newh[k]] = (int32_t)hg.size();
-      hg.push_back(newh[k]);
-    }
-    std::array<int32_t, 8> ec;
-    for (int c = 0; c < 8; ++c) {
-      const int32_t j = enode[8 * e + c] & kIdxMask;
-      ec[c] = j < N ? slot_n[j] : ~slot_h[j - (int32_t)N];
-    }
-    ecorner.push_back(ec);
+    P.rec.insert(P.rec.end(), p->rec.begin(), p->rec.end());
+    p.reset();
   }
-  close(n);
   P.elem.push_back((int32_t)n);
-  P.slot.push_back((int32_t)P.node.size());
-  for (auto& id : P.node)
-    if (id >= 0 && count[id & kIdxMask & ~kDirBit] == 1) id |= kOwnBit;
+  parallel_for((int64_t)P.head.size(), [&](int64_t b, int64_t e) {
+    for (int64_t k = b; k < e; ++k) {
+      uint32_t* r = &P.rec[4 * (size_t)P.head[k].x];
+      for (uint32_t i = 0; i < (P.head[k].y & 0xffffu); ++i)
+        if (count[r[i] & kNodeMask] == 1) r[i] |= (uint32_t)kOwnBit;
+    }
+  });
 }
 
 chns_status build_mesh(const uint32_t* anchors, const uint8_t* levels, int64_t n,
@@ -438,7 +606,7 @@ chns_status build_mesh(const uint32_t* anchors, const uint8_t* levels, int64_t n
 
   // ---- patches (CTA-level gather / scatter)
   PatchTables P;
-  build_patches(n, N, enode, hang, levels, P);
+  build_patches(n, N, anchors, enode, hang, levels, P);
 
   // ---- upload
   m->d.n_elem = n;
@@ -471,26 +639,19 @@ chns_status build_mesh(const uint32_t* anchors, const uint8_t* levels, int64_t n
     CHNS_CUDA(cudaStreamSynchronize(stream));
   }
   {
-    const int64_t np = (int64_t)P.nreg.size();
+    const int64_t np = (int64_t)P.head.size();
     m->d.n_patch = np;
-    m->n_slots = (int64_t)P.node.size();
     CHNS_CUDA(cudaMalloc(&m->d_patch_elem, (np + 1) * sizeof(int32_t)));
-    CHNS_CUDA(cudaMalloc(&m->d_patch_slot, (np + 1) * sizeof(int32_t)));
-    CHNS_CUDA(cudaMalloc(&m->d_patch_nreg, np * sizeof(int32_t)));
-    CHNS_CUDA(cudaMalloc(&m->d_slot_node, P.node.size() * sizeof(int32_t)));
-    CHNS_CUDA(cudaMalloc(&m->d_slot_par, P.par.size() * sizeof(ushort4)));
+    CHNS_CUDA(cudaMalloc(&m->d_patch_head, np * sizeof(uint4)));
+    CHNS_CUDA(cudaMalloc(&m->d_rec, P.rec.size() * sizeof(uint32_t)));
     CHNS_CUDA(cudaMalloc(&m->d_eloc, (size_t)n * sizeof(uint4)));
     CHNS_CUDA(cudaMemcpy(m->d_patch_elem, P.elem.data(), (np + 1) * sizeof(int32_t), cudaMemcpyHostToDevice));
-    CHNS_CUDA(cudaMemcpy(m->d_patch_slot, P.slot.data(), (np + 1) * sizeof(int32_t), cudaMemcpyHostToDevice));
-    CHNS_CUDA(cudaMemcpy(m->d_patch_nreg, P.nreg.data(), np * sizeof(int32_t), cudaMemcpyHostToDevice));
-    CHNS_CUDA(cudaMemcpy(m->d_slot_node, P.node.data(), P.node.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
-    CHNS_CUDA(cudaMemcpy(m->d_slot_par, P.par.data(), P.par.size() * sizeof(ushort4), cudaMemcpyHostToDevice));
+    CHNS_CUDA(cudaMemcpy(m->d_patch_head, P.head.data(), np * sizeof(uint4), cudaMemcpyHostToDevice));
+    CHNS_CUDA(cudaMemcpy(m->d_rec, P.rec.data(), P.rec.size() * sizeof(uint32_t), cudaMemcpyHostToDevice));
     CHNS_CUDA(cudaMemcpy(m->d_eloc, P.eloc.data(), (size_t)n * sizeof(uint4), cudaMemcpyHostToDevice));
     m->d.patch_elem = m->d_patch_elem;
-    m->d.patch_slot = m->d_patch_slot;
-    m->d.patch_nreg = m->d_patch_nreg;
-    m->d.slot_node = m->d_slot_node;
-    m->d.slot_par = m->d_slot_par;
+    m->d.patch_head = m->d_patch_head;
+    m->d.rec = m->d_rec;
     m->d.eloc = m->d_eloc;
   }
   {

@@ -89,7 +89,6 @@ struct PoissonK {
   // CTAs of the patch apply resident per SM that the register allocation must allow (FP32: 6,
   // i.e. at most 42 registers; FP64: 3)
   static constexpr int MIN_CTAS = sizeof(T) == 4 ? 6 : 3;
-  static constexpr int STREAM_CTAS = sizeof(T) == 4 ? 6 : 0;  // persistent apply (0: not used)
   static constexpr int NC = 1;
   static constexpr bool DIR = false;
   static constexpr bool DIAG_PER_COMP = false;
@@ -124,7 +123,6 @@ template <class T, class C>
 struct MassK {
   static constexpr bool QDATA = false;
   static constexpr int MIN_CTAS = sizeof(T) == 4 ? 5 : 3;
-  static constexpr int STREAM_CTAS = sizeof(T) == 4 ? 3 : 0;  // persistent apply (0: not used)
   static constexpr int NC = 3;
   static constexpr bool DIR = true;
   static constexpr bool DIAG_PER_COMP = false;
@@ -165,7 +163,6 @@ template <class T, class C>
 struct ShiftK {
   static constexpr bool QDATA = false;
   static constexpr int MIN_CTAS = sizeof(T) == 4 ? 6 : 3;
-  static constexpr int STREAM_CTAS = sizeof(T) == 4 ? 6 : 0;  // persistent apply (FP32)
   static constexpr int NC = 1;
   static constexpr bool DIR = false;
   static constexpr bool DIAG_PER_COMP = false;
@@ -254,7 +251,6 @@ template <class T, class C>
 struct ChK {
   static constexpr bool QDATA = false;
   static constexpr int MIN_CTAS = sizeof(T) == 4 ? 4 : 1;
-  static constexpr int STREAM_CTAS = 0;  // persistent apply (0: not used)
   static constexpr int NC = 2;
   static constexpr bool DIR = false;
   static constexpr bool DIAG_PER_COMP = true;
@@ -422,7 +418,6 @@ struct MomK {
   static constexpr bool QDATA = false;
   // FP32: two CTAs per SM (at most 128 registers) instead of the one that 217 registers allow
   static constexpr int MIN_CTAS = sizeof(T) == 4 ? 2 : 1;
-  static constexpr int STREAM_CTAS = 0;  // persistent apply (0: not used)
   static constexpr int NC = 3;
   static constexpr bool DIR = true;
   static constexpr bool DIAG_PER_COMP = false;
@@ -525,7 +520,6 @@ template <class T, class C>
 struct MomQK {
   static constexpr bool QDATA = true;
   static constexpr int MIN_CTAS = sizeof(T) == 4 ? 2 : 1;
-  static constexpr int STREAM_CTAS = 0;  // persistent apply (0: not used)
   static constexpr int NC = 3;
   static constexpr bool DIR = true;
   static constexpr bool DIAG_PER_COMP = false;
