@@ -10,6 +10,7 @@
 #pragma once
 
 #include "dfloat.cuh"
+#include "f32x2.cuh"
 #include "internal.h"
 
 namespace chns {
@@ -92,10 +93,56 @@ inline DevParams make_dev_params(const chns_params& p) {
 template <class T>
 using AccumT = typename std::conditional<std::is_same<T, DF>::value, double, T>::type;
 
+// GB300 executes two FP64 operations per clock and SM against 128 in FP32, and comparisons count:
+// the FP64 helpers below use integer operations where they can.
+
+// |v| < 1
+template <class T>
+__device__ __forceinline__ bool inside1(T v) {
+  if constexpr (std::is_same<T, double>::value)
+    return (__double2hiint(v) & 0x7fffffff) < 0x3ff00000;
+  else
+    return v < T(1) && v > T(-1);
+}
+// v clamped to [-1, 1]; NaN stays
 template <class T>
 __device__ __forceinline__ T clamp1(T v) {
-  return v > T(1) ? T(1) : (v < T(-1) ? T(-1) : v);
+  if constexpr (std::is_same<T, double>::value) {
+    const int hi = __double2hiint(v);
+    const bool out = (unsigned)((hi & 0x7fffffff) - 0x3ff00000) <= 0x40000000u;  // 1 <= |v| <= inf
+    return out ? __hiloint2double((hi & (int)0x80000000) | 0x3ff00000, 0) : v;
+  } else {
+    return v > T(1) ? T(1) : (v < T(-1) ? T(-1) : v);
+  }
 }
+
+// a b + c in one rounding where the type has it
+__device__ __forceinline__ float mad(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ double mad(double a, double b, double c) { return ::fma(a, b, c); }
+__device__ __forceinline__ DF mad(DF a, DF b, DF c) { return a * b + c; }
+
+// 1/x for normal x: the hardware estimate y (about 20 bits) and one third-order step
+// y (1 + e + e^2), e = 1 - x y (Householder's method): three operations, one ulp
+__device__ __forceinline__ double recip(double x) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = ::fma(-x, y, 1.0);
+  return ::fma(y, ::fma(e, e, e), y);
+}
+__device__ __forceinline__ float recip(float x) { return __fdividef(1.f, x); }  // a few ulp
+__device__ __forceinline__ DF recip(DF x) { return df_recip(x); }
+
+// 1/sqrt(x) for normal x > 0 (0 for infinity), in FP64 likewise: y (1 + e/2 + 3 e^2 / 8),
+// e = 1 - x y^2
+__device__ __forceinline__ double inv_sqrt(double x) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = ::fma(-x * y, y, 1.0);
+  const double z = ::fma(y * e, ::fma(0.375, e, 0.5), y);
+  return __double2hiint(x) == 0x7ff00000 ? 0.0 : z;
+}
+__device__ __forceinline__ float inv_sqrt(float x) { return rsqrt(x); }
+__device__ __forceinline__ DF inv_sqrt(DF x) { return rsqrt(x); }
 
 // ---- loads with conversion from the storage type
 template <class T>
@@ -214,175 +261,189 @@ __device__ __forceinline__ void scatter(const MeshDev& m, const int idx[8], cons
 }
 
 // ---- sum-factorised Q1 kernels
-// o0 = W0 a + W1 b and o1 = W1 a + W0 b, written with W0 = 1 - W1 as a + W1 (b - a) and
-// b - W1 (b - a): one subtraction and two fused multiply-adds.
+// 1D interpolation to the Gauss points and its transpose (B is symmetric), divided by W0:
+// o0 = a + r b, o1 = r a + b with r = W1 / W0, two operations. Every axis interpolated leaves a
+// factor gauss_w<T>() to the caller, who folds it into a constant: that of the rounded ratio,
+// 1 / (1 + r), so that constants are reproduced to the last rounding.
+constexpr double kRat = 0.26794919243112270647;
 template <class T>
-__device__ __forceinline__ void interp1(T a, T b, T& o0, T& o1) {
-  const T d = b - a;
-  o0 = a + T(kW1) * d;
-  o1 = b - T(kW1) * d;
+constexpr double gauss_w() {
+  if constexpr (std::is_same<T, double>::value || std::is_same<T, DF>::value)
+    return kW0;
+  else
+    return 1.0 / (1.0 + (double)(float)kRat);
 }
-
-// 2D interpolation of 4 values (i0 + 2 i1) to the 4 Gauss points; B symmetric => self-transpose.
 template <class T>
-__device__ __forceinline__ void interp2(const T in[4], T out[4]) {
-  T t[4];
-  interp1(in[0], in[1], t[0], t[1]);
-  interp1(in[2], in[3], t[2], t[3]);
-  interp1(t[0], t[2], out[0], out[2]);
-  interp1(t[1], t[3], out[1], out[3]);
+__device__ __forceinline__ void it(T a, T b, T& o0, T& o1) {
+  o0 = mad(T(kRat), b, a);
+  o1 = mad(T(kRat), a, b);
+}
+// Normalised form, o0 = a + W1 (b - a) and o1 = b - W1 (b - a): one more operation; reproduces
+// constants exactly and halves the rounding error of a chain of them.
+template <class T>
+__device__ __forceinline__ void itn(T a, T b, T& o0, T& o1) {
+  const T d = b - a;
+  o0 = mad(T(kW1), d, a);
+  o1 = mad(T(-kW1), d, b);
+}
+template <bool NORM, class T>
+__device__ __forceinline__ void interp(T a, T b, T& o0, T& o1) {
+  if constexpr (NORM)
+    itn(a, b, o0, o1);
+  else
+    it(a, b, o0, o1);
 }
 
 // 3D interpolation of corner values to the 8 Gauss points (self-transpose).
-template <class T>
+template <bool NORM, class T>
 __device__ __forceinline__ void interp3(const T u[8], T v[8]) {
   T t[8], s[8];
 #pragma unroll
-  for (int j = 0; j < 4; ++j) interp1(u[2 * j], u[2 * j + 1], t[2 * j], t[2 * j + 1]);
+  for (int j = 0; j < 4; ++j) interp<NORM>(u[2 * j], u[2 * j + 1], t[2 * j], t[2 * j + 1]);
 #pragma unroll
   for (int z = 0; z < 2; ++z)
 #pragma unroll
-    for (int x = 0; x < 2; ++x) interp1(t[x + 4 * z], t[x + 2 + 4 * z], s[x + 4 * z], s[x + 2 + 4 * z]);
+    for (int x = 0; x < 2; ++x)
+      interp<NORM>(t[x + 4 * z], t[x + 2 + 4 * z], s[x + 4 * z], s[x + 2 + 4 * z]);
 #pragma unroll
-  for (int i = 0; i < 4; ++i) interp1(s[i], s[i + 4], v[i], v[i + 4]);
+  for (int i = 0; i < 4; ++i) interp<NORM>(s[i], s[i + 4], v[i], v[i + 4]);
 }
-
-// Reference-gradient data of an element: gx depends on (qy,qz) only, gy on (qx,qz), gz on (qx,qy);
-// each is the bilinear interpolation of the 4 edge differences along that axis. Physical
-// gradient = g / h (the factor 2/h of the Jacobian times the 1/2 of the 1D derivative).
+// 2D, 4 values (i0 + 2 i1)
 template <class T>
-__device__ __forceinline__ void grad_compact(const T u[8], T gx[4], T gy[4], T gz[4]) {
-  T d[4];
-#pragma unroll
-  for (int j = 0; j < 4; ++j) d[j] = u[2 * j + 1] - u[2 * j];  // j = y + 2z
-  interp2(d, gx);
-#pragma unroll
-  for (int z = 0; z < 2; ++z)
-#pragma unroll
-    for (int x = 0; x < 2; ++x) d[x + 2 * z] = u[x + 2 + 4 * z] - u[x + 4 * z];
-  interp2(d, gy);
-#pragma unroll
-  for (int j = 0; j < 4; ++j) d[j] = u[j + 4] - u[j];  // j = x + 2y
-  interp2(d, gz);
-}
-
-// Transpose of grad_compact for per-axis sums over the free Gauss coordinate:
-// r_a += sign(a_d) * interp2(S_d)[other bits of a] * scale_d.
-template <class T>
-__device__ __forceinline__ void grad_compact_T(const T sx[4], const T sy[4], const T sz[4],
-                                               const T sc[3], T r[8]) {
+__device__ __forceinline__ void interp2(const T in[4], T out[4]) {
   T t[4];
-  interp2(sx, t);
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    r[2 * j + 1] += sc[0] * t[j];
-    r[2 * j] -= sc[0] * t[j];
-  }
-  interp2(sy, t);
-#pragma unroll
-  for (int z = 0; z < 2; ++z)
-#pragma unroll
-    for (int x = 0; x < 2; ++x) {
-      r[x + 2 + 4 * z] += sc[1] * t[x + 2 * z];
-      r[x + 4 * z] -= sc[1] * t[x + 2 * z];
-    }
-  interp2(sz, t);
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    r[j + 4] += sc[2] * t[j];
-    r[j] -= sc[2] * t[j];
-  }
+  it(in[0], in[1], t[0], t[1]);
+  it(in[2], in[3], t[2], t[3]);
+  it(t[0], t[2], out[0], out[2]);
+  it(t[1], t[3], out[1], out[3]);
 }
 
-// Physical gradient components at Gauss point Q from the compact data of grad_compact:
-// d/dx at (qy, qz) = gx[Q >> 1] / h_x, d/dy at (qx, qz) = gy[(Q & 1) + 2 (Q >> 2)] / h_y,
-// d/dz at (qx, qy) = gz[Q & 3] / h_z.
-__device__ __forceinline__ constexpr int gxi(int Q) { return Q >> 1; }
-__device__ __forceinline__ constexpr int gyi(int Q) { return (Q & 1) + 2 * (Q >> 2); }
-__device__ __forceinline__ constexpr int gzi(int Q) { return Q & 3; }
-
-// r_a += sum_q grad N_a(q) . V_q for per-point vectors V[d][q] (physical units, quadrature
-// weights and coefficients included): the x component of grad N_a does not depend on qx, so V_x
-// is first summed over qx (likewise y, z), then the compact transpose applies.
+// Compact gradient data of an element: the x difference depends on (qy, qz) only, and so on; each
+// is the bilinear interpolation of the 4 edge differences along its axis. True values are these
+// times gauss_w^2 / h_d.
 template <class T>
-__device__ __forceinline__ void grad_T(const T V[3][8], const Geo<T>& g, T r[8]) {
-  T sx[4], sy[4], sz[4];
+struct GradC {
+  T x[4], y[4], z[4];  // [qy + 2 qz], [qx + 2 qz], [qx + 2 qy]
+  __device__ __forceinline__ void eval(const T u[8]) {
+    T d[4];
 #pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    sx[j] = V[0][2 * j] + V[0][2 * j + 1];
-    sz[j] = V[2][j] + V[2][j + 4];
+    for (int j = 0; j < 4; ++j) d[j] = u[2 * j + 1] - u[2 * j];
+    interp2(d, x);
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+#pragma unroll
+      for (int i = 0; i < 2; ++i) d[i + 2 * k] = u[i + 2 + 4 * k] - u[i + 4 * k];
+    interp2(d, y);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) d[j] = u[j + 4] - u[j];
+    interp2(d, z);
   }
+  // physical gradients (c_d = gauss_w^2 / h_d, times whatever the caller folds in)
+  __device__ __forceinline__ void eval(const T u[8], const T c[3]) {
+    eval(u);
 #pragma unroll
-  for (int z = 0; z < 2; ++z)
-#pragma unroll
-    for (int x = 0; x < 2; ++x) sy[x + 2 * z] = V[1][x + 4 * z] + V[1][x + 2 + 4 * z];
-  const T sc[3] = {g.ih[0], g.ih[1], g.ih[2]};
-  grad_compact_T(sx, sy, sz, sc, r);
-}
-
-// ---- per-quadrature-point evaluation (direct; used by the multi-field operators)
-__device__ __forceinline__ constexpr double b1(int a, int q) { return a == q ? kW0 : kW1; }
-__device__ __forceinline__ constexpr double sg(int a) { return a ? 1.0 : -1.0; }
-
-// N_a(q), and the reference factor of dN_a/dx_d(q) * h_d  (= sign * product of the other two B)
-__device__ __forceinline__ constexpr double Nq(int a, int q) {
-  return b1(a & 1, q & 1) * b1((a >> 1) & 1, (q >> 1) & 1) * b1((a >> 2) & 1, (q >> 2) & 1);
-}
-__device__ __forceinline__ constexpr double dNq(int a, int q, int d) {
-  return d == 0 ? sg(a & 1) * b1((a >> 1) & 1, (q >> 1) & 1) * b1((a >> 2) & 1, (q >> 2) & 1)
-       : d == 1 ? sg((a >> 1) & 1) * b1(a & 1, q & 1) * b1((a >> 2) & 1, (q >> 2) & 1)
-                : sg((a >> 2) & 1) * b1(a & 1, q & 1) * b1((a >> 1) & 1, (q >> 1) & 1);
-}
-
-// value and physical gradient at quadrature point Q of an element field u[8]
-template <int Q, class T>
-__device__ __forceinline__ void vg_at(const T u[8], const Geo<T>& g, T& v, T gr[3]) {
-  v = T(0);
-  gr[0] = gr[1] = gr[2] = T(0);
-#pragma unroll
-  for (int a = 0; a < 8; ++a) {
-    v += T(Nq(a, Q)) * u[a];
-    gr[0] += T(dNq(a, Q, 0)) * u[a];
-    gr[1] += T(dNq(a, Q, 1)) * u[a];
-    gr[2] += T(dNq(a, Q, 2)) * u[a];
+    for (int j = 0; j < 4; ++j) {
+      x[j] *= c[0];
+      y[j] *= c[1];
+      z[j] *= c[2];
+    }
   }
-  gr[0] *= g.ih[0];
-  gr[1] *= g.ih[1];
-  gr[2] *= g.ih[2];
-}
+  // component d at Gauss point q
+  __device__ __forceinline__ T at(int q, int d) const {
+    return d == 0 ? x[q >> 1] : d == 1 ? y[(q & 1) + 2 * (q >> 2)] : z[q & 3];
+  }
+  // adds (FIRST: sets) the component d of a per-point vector at Gauss point q: the data whose
+  // transpose is the sum over the points of grad N_a . V
+  __device__ __forceinline__ void sum(int q, int d, T v) {
+    T& s = d == 0 ? x[q >> 1] : d == 1 ? y[(q & 1) + 2 * (q >> 2)] : z[q & 3];
+    const bool first = d == 0 ? !(q & 1) : d == 1 ? !(q & 2) : !(q & 4);
+    s = first ? v : s + v;
+  }
+  // r_a += sum_d sc_d (transpose of eval)
+  __device__ __forceinline__ void transpose(const T sc[3], T r[8]) const {
+    T t[4];
+    interp2(x, t);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      r[2 * j + 1] = mad(sc[0], t[j], r[2 * j + 1]);
+      r[2 * j] = mad(-sc[0], t[j], r[2 * j]);
+    }
+    interp2(y, t);
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        r[i + 2 + 4 * k] = mad(sc[1], t[i + 2 * k], r[i + 2 + 4 * k]);
+        r[i + 4 * k] = mad(-sc[1], t[i + 2 * k], r[i + 4 * k]);
+      }
+    interp2(z, t);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      r[j + 4] = mad(sc[2], t[j], r[j + 4]);
+      r[j] = mad(-sc[2], t[j], r[j]);
+    }
+  }
+};
 
-template <int Q, class T>
-__device__ __forceinline__ T val_at(const T u[8]) {
-  T v = T(0);
+// One field of a constant-coefficient form on a box. The 2x2x2 Gauss rule is exact there and the
+// element matrices are Kronecker products of the 1D matrices m = h/6 [[2, 1], [1, 2]] and
+// k = 1/h [[1, -1], [-1, 1]]: with P(a, b) = (2a + b, a + 2b) and D(a, b) = (a - b, b - a) along
+// one axis, M_e u = V/216 Px B and K_e u = V/36 (Px (C / h_y^2 + E / h_z^2) + Dx B / h_x^2), where
+// B = Py Pz u, C = Dy Pz u, E = Py Dz u and V = h_x h_y h_z.
+template <class T>
+struct Kron {
+  T B[8], C[4], E[4];  // C at y = 0 [x + 2 z] (y = 1: its negative), E at z = 0 [x + 2 y] (likewise)
+  __device__ __forceinline__ void mass(const T u[8]) {
+    T p[8];
+    stage(u, p);
+  }
+  __device__ __forceinline__ void eval(const T u[8]) {
+    T p[8], w[4];
+    stage(u, p);
 #pragma unroll
-  for (int a = 0; a < 8; ++a) v += T(Nq(a, Q)) * u[a];
-  return v;
-}
+    for (int k = 0; k < 2; ++k)
+#pragma unroll
+      for (int i = 0; i < 2; ++i) C[i + 2 * k] = p[i + 4 * k] - p[i + 2 + 4 * k];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) w[j] = u[j] - u[j + 4];
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      E[i] = mad(T(2), w[i], w[i + 2]);
+      E[i + 2] = mad(T(2), w[i + 2], w[i]);
+    }
+  }
+  __device__ __forceinline__ T c_at(int a) const {
+    const T v = C[(a & 1) + 2 * (a >> 2)];
+    return a & 2 ? -v : v;
+  }
+  __device__ __forceinline__ T e_at(int a) const { return a & 4 ? -E[a & 3] : E[a & 3]; }
+  // r = Px S + cx Dx B (of this field)
+  __device__ __forceinline__ void finish(const T S[8], T cx, T r[8]) const {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const T d = B[2 * j] - B[2 * j + 1];
+      r[2 * j] = mad(cx, d, mad(T(2), S[2 * j], S[2 * j + 1]));
+      r[2 * j + 1] = mad(-cx, d, mad(T(2), S[2 * j + 1], S[2 * j]));
+    }
+  }
 
-// r_a += N_a(Q) s + grad N_a(Q) . V   (V already in physical units; scaled here by 1/h)
-template <int Q, class T>
-__device__ __forceinline__ void add_test(T r[8], T s, const T V[3], const Geo<T>& g) {
-  T vx = V[0] * g.ih[0], vy = V[1] * g.ih[1], vz = V[2] * g.ih[2];
+ private:
+  __device__ __forceinline__ void stage(const T u[8], T p[8]) {
 #pragma unroll
-  for (int a = 0; a < 8; ++a)
-    r[a] += T(Nq(a, Q)) * s + T(dNq(a, Q, 0)) * vx + T(dNq(a, Q, 1)) * vy + T(dNq(a, Q, 2)) * vz;
-}
-
-// Mixed second derivatives of the trilinear interpolant at Q: H_xy, H_xz, H_yz (pure ones vanish).
-template <int Q, class T>
-__device__ __forceinline__ void hess_at(const T u[8], const Geo<T>& g, T& hxy, T& hxz, T& hyz) {
-  const int qx = Q & 1, qy = (Q >> 1) & 1, qz = (Q >> 2) & 1;
-  T dxy[2], dxz[2], dyz[2];
+    for (int j = 0; j < 4; ++j) {
+      p[j] = mad(T(2), u[j], u[j + 4]);
+      p[j + 4] = mad(T(2), u[j + 4], u[j]);
+    }
 #pragma unroll
-  for (int z = 0; z < 2; ++z) dxy[z] = u[3 + 4 * z] - u[2 + 4 * z] - u[1 + 4 * z] + u[4 * z];
+    for (int k = 0; k < 2; ++k)
 #pragma unroll
-  for (int y = 0; y < 2; ++y) dxz[y] = u[5 + 2 * y] - u[4 + 2 * y] - u[1 + 2 * y] + u[2 * y];
-#pragma unroll
-  for (int x = 0; x < 2; ++x) dyz[x] = u[6 + x] - u[4 + x] - u[2 + x] + u[x];
-  hxy = (T(b1(0, qz)) * dxy[0] + T(b1(1, qz)) * dxy[1]) * g.ih[0] * g.ih[1];
-  hxz = (T(b1(0, qy)) * dxz[0] + T(b1(1, qy)) * dxz[1]) * g.ih[0] * g.ih[2];
-  hyz = (T(b1(0, qx)) * dyz[0] + T(b1(1, qx)) * dyz[1]) * g.ih[1] * g.ih[2];
-}
+      for (int i = 0; i < 2; ++i) {
+        const int a = i + 4 * k, b = a + 2;
+        B[a] = mad(T(2), p[a], p[b]);
+        B[b] = mad(T(2), p[b], p[a]);
+      }
+  }
+};
 
 // Compile-time loop over the 8 quadrature points.
 template <int Q = 0, class F>

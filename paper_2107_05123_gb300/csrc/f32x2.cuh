@@ -1,7 +1,7 @@
 // Pairs of FP32 numbers in one 64-bit register pair. The packed instructions of sm_10x (FADD2,
 // FMUL2, FFMA2) do two FP32 operations, each rounded as the scalar one, in one issue slot; the
 // FP32 applies are bound by instruction issue, so their element arithmetic runs on two elements
-// at a time. The helpers below exist for float and F2 so that one source serves both.
+// at a time.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -18,8 +18,7 @@ struct __align__(8) F2 {
 __device__ __forceinline__ float2 raw(F2 a) { return make_float2(a.x, a.y); }
 __device__ __forceinline__ F2 from_raw(float2 a) { return F2(a.x, a.y); }
 
-__device__ __forceinline__ float vfma(float a, float b, float c) { return fmaf(a, b, c); }
-__device__ __forceinline__ F2 vfma(F2 a, F2 b, F2 c) {
+__device__ __forceinline__ F2 mad(F2 a, F2 b, F2 c) {
   return from_raw(__ffma2_rn(raw(a), raw(b), raw(c)));
 }
 __device__ __forceinline__ F2 operator+(F2 a, F2 b) { return from_raw(__fadd2_rn(raw(a), raw(b))); }

@@ -47,229 +47,239 @@ k_residual_ch(MeshDev m, DevParams p, const double* __restrict__ phi, const doub
   for (int i = 0; i < 8; ++i) mt[i] = A(0.5) * (a[i] + b[i]);
 #pragma unroll
   for (int d = 0; d < 3; ++d) gather<A, false>(m, idx, u.c[d], ue[d]);
-  // sum-factorised: values at the Gauss points by interp3, gradients by grad_compact, and the
-  // transposes interp3 / grad_T on the per-point terms
-  A r0[8], r1[8];
-  const A J = g.detJ, kmu = k.inv_pecn, c2 = k.cn2;
-  A pv[8], mv[8], s[8], V[3][8];
-  interp3(pt, pv);
-  interp3(mt, mv);
-#pragma unroll
-  for (int q = 0; q < 8; ++q) s[q] = J * (pv[q] * pv[q] * pv[q] - pv[q] - mv[q]);
-  interp3(s, r1);
+  // the constant-coefficient terms as Kronecker products (Kron), psi' and the advection at the
+  // Gauss points
+  constexpr double w = gauss_w<A>(), w3 = w * w * w;
+  const A J = g.detJ, Vol = A(8) * J, cm = Vol * A(1.0 / 216.0), ks = Vol * A(1.0 / 36.0);
+  const A kh[3] = {ks * g.ih[0] * g.ih[0], ks * g.ih[1] * g.ih[1], ks * g.ih[2] * g.ih[2]};
+  A r0[8], r1[8], s[8];
   {
-    A gx[4], gy[4], gz[4];
-    grad_compact(pt, gx, gy, gz);
-    const A jc = J * c2;
+    Kron<A> kd, kp, kq;
+    kd.mass(dp);
+    kq.eval(mt);
+    const A cy = k.inv_pecn * kh[1], cz = k.inv_pecn * kh[2];
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      V[0][q] = jc * gx[gxi(q)] * g.ih[0];
-      V[1][q] = jc * gy[gyi(q)] * g.ih[1];
-      V[2][q] = jc * gz[gzi(q)] * g.ih[2];
-    }
-    grad_T(V, g, r1);
+    for (int i = 0; i < 8; ++i) s[i] = mad(cm, kd.B[i], mad(cy, kq.c_at(i), cz * kq.e_at(i)));
+    kq.finish(s, k.inv_pecn * kh[0], r0);
+    kp.eval(pt);
+    const A py = k.cn2 * kh[1], pz = k.cn2 * kh[2];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) s[i] = mad(-cm, kq.B[i], mad(py, kp.c_at(i), pz * kp.e_at(i)));
+    kp.finish(s, k.cn2 * kh[0], r1);
   }
-  interp3(dp, s);
+  A pv[8];
+  interp3<false>(pt, pv);
+  // (q, phi^3 - phi) from the unnormalised values: w^3 (test) (w^9 p^3 - w^3 p)
+  const A c1 = J * A(w3 * w3), c3 = c1 * A(w3 * w3);
 #pragma unroll
-  for (int q = 0; q < 8; ++q) s[q] = s[q] * J;
-  interp3(s, r0);
-  {
-    A gx[4], gy[4], gz[4], uq[8];
-    grad_compact(mt, gx, gy, gz);
+  for (int q = 0; q < 8; ++q) s[q] = mad(c3 * pv[q], pv[q], -c1) * pv[q];
+  A t[8];
+  interp3<false>(s, t);
 #pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      interp3(ue[d], uq);
+  for (int i = 0; i < 8; ++i) r1[i] += t[i];
+  GradC<A> d;
 #pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        const A gm = d == 0 ? gx[gxi(q)] : d == 1 ? gy[gyi(q)] : gz[gzi(q)];
-        V[d][q] = J * (kmu * gm * g.ih[d] - uq[q] * pv[q]);
-      }
-    }
-    grad_T(V, g, r0);
+  for (int c = 0; c < 3; ++c) {
+    interp3<false>(ue[c], t);
+#pragma unroll
+    for (int q = 0; q < 8; ++q) d.sum(q, c, t[q] * pv[q]);
   }
+  const A ca = J * A(-w3 * w3 * w * w);
+  const A sc[3] = {ca * g.ih[0], ca * g.ih[1], ca * g.ih[2]};
+  d.transpose(sc, r0);
   scatter<A, false>(m, idx, r0, f);
   scatter<A, false>(m, idx, r1, f + m.n_nodes);
 }
 
-// Forcing d_j(d_i phi d_j phi) of the trilinear interpolant at Q (pure second derivatives vanish
-// on box elements): F_i = sum_{j != i} H_ij d_j phi.
-template <int Q, class A>
-__device__ __forceinline__ void forcing_at(const A pe[8], const Geo<A>& g, const A gp[3], A F[3]) {
-  A hxy, hxz, hyz;
-  hess_at<Q>(pe, g, hxy, hxz, hyz);
-  F[0] = hxy * gp[1] + hxz * gp[2];
-  F[1] = hxy * gp[0] + hyz * gp[2];
-  F[2] = hxz * gp[0] + hyz * gp[1];
-}
-
-// rho g_i / Fr for the component i (g_hat = (0, -1, 0))
+// Mixed second derivatives of the trilinear interpolant (the pure ones vanish on box elements):
+// H_xy depends on qz only, H_xz on qy, H_yz on qx. Forcing d_j(d_i phi d_j phi) at a point:
+// F_i = sum_{j != i} H_ij d_j phi.
 template <class A>
-__device__ __forceinline__ A gravity(const A& rho, const PrmT<A>& k, int i) {
-  return ghat(i) == 0 ? A(0) : -(rho * k.inv_fr);
-}
+struct Forcing {
+  A xy[2], xz[2], yz[2];
+  __device__ __forceinline__ Forcing(const A u[8], const Geo<A>& g, const A& scale) {
+    constexpr double w = gauss_w<A>();
+    const A c = A(w) * scale;
+    it(u[3] - u[2] - u[1] + u[0], u[7] - u[6] - u[5] + u[4], xy[0], xy[1]);
+    it(u[5] - u[4] - u[1] + u[0], u[7] - u[6] - u[3] + u[2], xz[0], xz[1]);
+    it(u[6] - u[4] - u[2] + u[0], u[7] - u[5] - u[3] + u[1], yz[0], yz[1]);
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      xy[i] *= c * g.ih[0] * g.ih[1];
+      xz[i] *= c * g.ih[0] * g.ih[2];
+      yz[i] *= c * g.ih[1] * g.ih[2];
+    }
+  }
+  // component i at point q, times the scale, added to v
+  __device__ __forceinline__ A add(int q, int i, const A gp[3], A v) const {
+    const A a = xy[q >> 2], b = xz[q >> 1 & 1], c = yz[q & 1];
+    return i == 0   ? mad(a, gp[1], mad(b, gp[2], v))
+           : i == 1 ? mad(a, gp[0], mad(c, gp[2], v))
+                    : mad(b, gp[0], mad(c, gp[1], v));
+  }
+};
 
 // ---- velocity-prediction right-hand side (Def. weak_VMS_disc), per component i:
 //   (w, rho u_i/dt) - 1/2 (w, rho u.grad u_i) - 1/(2Pe) (w, J.grad u_i) - 1/(2Re) (grad w, eta grad u_i)
 //   + Cn/We (d_j w, d_i phi d_j phi) - (w, d_i p) + (w, rho g_i/Fr) - (grad w . t, R0_i)
 // with R0_i the part of R_m that does not depend on v^{k+1}.
-// Sum-factorised: every field's values and gradients at the 8 Gauss points come from interp3 /
-// grad_compact, the per-point coefficients (tau_m and the advection and stabilisation vectors)
-// are formed once per point, and each component's test-function sums are the transposes interp3
-// and grad_T of its per-point terms.
-template <class A>
-struct MomPt {  // per-point data shared by the three components
-  A a0, b[3], bp[3], e, t[3], rho, gphi[3], F[3], pg[3];
-};
-
+// Every field's values and gradients at the 8 Gauss points come from interp3 / GradC. For each point
+// the coefficients (tau_m and the advection and stabilisation vectors) are formed once and the
+// three components' terms take the place of their values and sum up in compact gradient data; the
+// transposes follow.
 template <class A>
 __global__ void __launch_bounds__(kRhsThreads)
 k_rhs_momentum(MeshDev m, DevParams p, CoefArgs<double> cf, Ptr3 uk,
                const double* __restrict__ pk, double* __restrict__ b) {
   const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (e >= m.n_elem) return;
+  constexpr double w = gauss_w<A>();
   const PrmT<A>& k = p.get<A>();
   int idx[8];
   load_corners(m, e, idx);
   const Geo<A> g = geometry<A>(m, e);
-  const A J = g.detJ, cw = k.cw;
-  MomPt<A> c[8];
+  const A J = g.detJ, w3 = A(w * w * w), j3 = J * w3;
+  const A cg[3] = {A(w * w) * g.ih[0], A(w * w) * g.ih[1], A(w * w) * g.ih[2]};
+  const VmsElem<A> el(g, k);
+  VmsFields<A> f;
+  A pe[8];
+  gather<A, false>(m, idx, cf.phi, pe);
   {
-    A pe[8], ue[3][8], me[8], pp[8];
-    gather<A, false>(m, idx, cf.phi, pe);
+    A ue[3][8], me[8];
 #pragma unroll
     for (int d = 0; d < 3; ++d) gather<A, false>(m, idx, cf.u[d], ue[d]);
     gather<A, false>(m, idx, cf.mu, me);
-    gather<A, false>(m, idx, pk, pp);
-    QpField<A> fp, fm, fr;
-    fp.eval(pe);
-    fm.eval_grad(me);
-    fr.eval_grad(pp);
-    A uq[3][8];
-#pragma unroll
-    for (int d = 0; d < 3; ++d) interp3(ue[d], uq[d]);
-    for_qp([&](auto QC) {
-      constexpr int Q = decltype(QC)::value;
-      A gp[3], mg[3], uv[3];
-#pragma unroll
-      for (int d = 0; d < 3; ++d) {
-        gp[d] = fp.grad(Q, d, g);
-        mg[d] = fm.grad(Q, d, g);
-        uv[d] = uq[d][Q];
-      }
-      const VmsQ<A> v = vms_point(fp.v[Q], gp, mg, uv, g, p);
-      MomPt<A>& o = c[Q];
-      o.a0 = v.a0;
-      o.e = v.e;
-      o.rho = v.rho;
-#pragma unroll
-      for (int d = 0; d < 3; ++d) {
-        o.b[d] = v.b[d];
-        o.bp[d] = v.bp[d];
-        o.t[d] = v.t[d];
-        o.gphi[d] = v.gphi[d];
-        o.pg[d] = fr.grad(Q, d, g);
-      }
-      forcing_at<Q>(pe, g, v.gphi, o.F);
-    });
+    f.eval(pe, me, ue, g, k);
   }
-#pragma unroll 1
-  for (int i = 0; i < 3; ++i) {
-    A ui[8];
-    gather<A, false>(m, idx, uk.c[i], ui);
-    QpField<A> fu;
-    fu.eval(ui);
-    A s[8], V[3][8];
+  const Forcing<A> fo(pe, g, k.cw);
+  GradC<A> gpr, d[3], s[3];
+  A v[3][8];
+  {
+    A t[8];
+    gather<A, false>(m, idx, pk, t);
+    gpr.eval(t, cg);
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      const MomPt<A>& o = c[q];
-      const A v = fu.v[q];
-      const A vg[3] = {fu.grad(q, 0, g), fu.grad(q, 1, g), fu.grad(q, 2, g)};
-      const A grav = gravity(o.rho, k, i);
-      const A bdot = o.b[0] * vg[0] + o.b[1] * vg[1] + o.b[2] * vg[2];
-      const A bpdot = o.bp[0] * vg[0] + o.bp[1] * vg[1] + o.bp[2] * vg[2];
-      const A r0 = bpdot - o.a0 * v + cw * o.F[i] + o.pg[i] - grav;
-      const A fn = o.a0 * v - bdot - o.pg[i] + grav;
-      s[q] = J * fn;
-      const A cg = cw * o.gphi[i];
-#pragma unroll
-      for (int d = 0; d < 3; ++d) V[d][q] = J * (cg * o.gphi[d] - o.e * vg[d] - o.t[d] * r0);
+    for (int i = 0; i < 3; ++i) {
+      gather<A, false>(m, idx, uk.c[i], t);
+      interp3<false>(t, v[i]);
+      d[i].eval(t, cg);
     }
+  }
+  for_qp([&](auto QC) {
+    constexpr int Q = decltype(QC)::value;
+    const VmsQ<A> c = f.at(Q, el, k);
+    const A gp[3] = {f.gp.at(Q, 0), f.gp.at(Q, 1), f.gp.at(Q, 2)};
+    const A a0 = c.a0 * w3;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      const A vg[3] = {d[i].at(Q, 0), d[i].at(Q, 1), d[i].at(Q, 2)};
+      // the part without advection, shared by both sums: a0 v - p_i + rho g_i / Fr
+      A h = mad(a0, v[i][Q], -gpr.at(Q, i));
+      if (ghat(i) != 0) h = mad(-c.rho, k.inv_fr, h);
+      // R_0: b'.grad v + Cn/We F - h, and the tested value h - b.grad v
+      const A r0 = fo.add(Q, i, gp, mad(c.bp[0], vg[0], mad(c.bp[1], vg[1], mad(c.bp[2], vg[2], -h))));
+      v[i][Q] = j3 * mad(-c.b[0], vg[0], mad(-c.b[1], vg[1], mad(-c.b[2], vg[2], h)));
+      const A cp = k.cw * gp[i];
+#pragma unroll
+      for (int n = 0; n < 3; ++n)
+        s[i].sum(Q, n, mad(cp, gp[n], -mad(c.e, vg[n], c.t[n] * r0)));
+    }
+  });
+  const A sc[3] = {J * cg[0], J * cg[1], J * cg[2]};
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
     A r[8];
-    interp3(s, r);
-    grad_T(V, g, r);
+    interp3<false>(v[i], r);
+    s[i].transpose(sc, r);
     scatter<A, true>(m, idx, r, b + i * m.n_nodes);
   }
 }
 
-// Full R_m,i(v) at a point (Def. of R_m) with v~ = (v + u_k)/2, from the point values vv and
-// gradients vgr of v and ug of u_k (uv: u_k's values).
-template <class A>
-__device__ __forceinline__ void rm_point(const VmsQ<A>& c, const PrmT<A>& k, const A F[3],
-                                         const A pg[3], const A vv[3], const A vgr[3][3],
-                                         const A uv[3], const A ug[3][3], A R[3], A& div) {
-  div = vgr[0][0] + vgr[1][1] + vgr[2][2];
-#pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    A tg[3];
-#pragma unroll
-    for (int d = 0; d < 3; ++d) tg[d] = A(0.5) * (vgr[i][d] + ug[i][d]);
-    const A adv = c.uq[0] * tg[0] + c.uq[1] * tg[1] + c.uq[2] * tg[2];
-    const A jdv = c.J[0] * tg[0] + c.J[1] * tg[1] + c.J[2] * tg[2];
-    const A edv = c.ge[0] * tg[0] + c.ge[1] * tg[1] + c.ge[2] * tg[2];
-    R[i] = c.rho * (vv[i] - uv[i]) * k.idt + c.rho * adv + jdv * k.inv_pe + k.cw * F[i] + pg[i] -
-           edv * k.inv_re - gravity(c.rho, k, i);
-  }
-}
-
-// The fields of the pressure-Poisson and velocity-update right-hand sides at the 8 Gauss points.
+// The fields of the pressure-Poisson and velocity-update right-hand sides at the 8 Gauss points:
+// v and the differences v - u_k, the gradients of v~ = (v + u_k)/2, and of p_k.
 template <class A>
 struct ProjFields {
-  QpField<A> fp, fm, fr, fv[3], fu[3];
-  A uq[3][8];
+  VmsFields<A> f;
+  GradC<A> gpr, gt[3];
+  A dv[3][8], vv[3][8];  // (v - u_k)/dt without gauss_w^3; v likewise
+  A div[8];
+  A pe[8];
   __device__ __forceinline__ void load(const MeshDev& m, const int idx[8],
                                        const CoefArgs<double>& cf, const Ptr3& v, const Ptr3& uk,
-                                       const double* pk, A pe[8]) {
-    A t[8];
+                                       const double* pk, const Geo<A>& g, const PrmT<A>& k) {
+    constexpr double w = gauss_w<A>();
+    const A cg[3] = {A(w * w) * g.ih[0], A(w * w) * g.ih[1], A(w * w) * g.ih[2]};
+    const A ch[3] = {A(0.5) * cg[0], A(0.5) * cg[1], A(0.5) * cg[2]};
+    A t[8], u[8];
     gather<A, false>(m, idx, cf.phi, pe);
-    fp.eval(pe);
-    gather<A, false>(m, idx, cf.mu, t);
-    fm.eval_grad(t);
-    gather<A, false>(m, idx, pk, t);
-    fr.eval_grad(t);
+    {
+      A ue[3][8];
 #pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      gather<A, false>(m, idx, cf.u[d], t);
-      interp3(t, uq[d]);
-      gather<A, false>(m, idx, v.c[d], t);
-      fv[d].eval(t);
-      gather<A, false>(m, idx, uk.c[d], t);
-      fu[d].eval(t);
+      for (int d = 0; d < 3; ++d) gather<A, false>(m, idx, cf.u[d], ue[d]);
+      gather<A, false>(m, idx, cf.mu, t);
+      f.eval(pe, t, ue, g, k);
+    }
+    gather<A, false>(m, idx, pk, t);
+    gpr.eval(t, cg);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      gather<A, false>(m, idx, v.c[i], t);
+      gather<A, false>(m, idx, uk.c[i], u);
+      interp3<false>(t, vv[i]);
+      axis_gradient(t, i, cg[i]);
+      A a[8];
+#pragma unroll
+      for (int n = 0; n < 8; ++n) a[n] = t[n] + u[n];
+      gt[i].eval(a, ch);
+#pragma unroll
+      for (int n = 0; n < 8; ++n) a[n] = (t[n] - u[n]) * k.idt;
+      interp3<false>(a, dv[i]);
     }
   }
-  // the coefficients, forcing, grad p_k and R_m at point Q
-  template <int Q>
-  __device__ __forceinline__ VmsQ<A> at(const A pe[8], const Geo<A>& g, const DevParams& p,
-                                        A pg[3], A R[3], A vv[3], A& div) const {
-    A gp[3], mg[3], uv0[3], vgr[3][3], ug[3][3], uv[3];
+  // R_m,i at point q (Def. of R_m)
+  __device__ __forceinline__ A residual(int q, int i, const VmsQ<A>& c, const A adv[3],
+                                        const A gp[3], const Forcing<A>& fo,
+                                        const PrmT<A>& k) const {
+    constexpr double w = gauss_w<A>();
+    A r = mad(c.rho * A(w * w * w), dv[i][q], gpr.at(q, i));
+#pragma unroll
+    for (int d = 0; d < 3; ++d) r = mad(adv[d], gt[i].at(q, d), r);
+    if (ghat(i) != 0) r = mad(c.rho, k.inv_fr, r);
+    return fo.add(q, i, gp, r);
+  }
+  // coefficients, advection vector rho u + J/Pe - grad eta/Re = 2 b', and grad phi~ of point q
+  __device__ __forceinline__ VmsQ<A> at(int q, const VmsElem<A>& el, const PrmT<A>& k, A adv[3],
+                                        A gp[3]) const {
+    const VmsQ<A> c = f.at(q, el, k);
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
-      gp[d] = fp.grad(Q, d, g);
-      mg[d] = fm.grad(Q, d, g);
-      uv0[d] = uq[d][Q];
-      pg[d] = fr.grad(Q, d, g);
-      vv[d] = fv[d].v[Q];
-      uv[d] = fu[d].v[Q];
+      gp[d] = f.gp.at(q, d);
+      adv[d] = A(2) * c.bp[d];
+    }
+    return c;
+  }
+
+ private:
+  // div += the axis-i derivative of t, at the 8 points
+  __device__ __forceinline__ void axis_gradient(const A t[8], int i, const A& c) {
+    A e[4], o[4];
 #pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        vgr[d][k] = fv[d].grad(Q, k, g);
-        ug[d][k] = fu[d].grad(Q, k, g);
+    for (int j = 0; j < 4; ++j) {
+      const int lo = i == 0 ? 2 * j : i == 1 ? (j & 1) + 4 * (j >> 1) : j;
+      e[j] = t[lo + (1 << i)] - t[lo];
+    }
+    interp2(e, o);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int lo = i == 0 ? 2 * j : i == 1 ? (j & 1) + 4 * (j >> 1) : j;
+      if (i == 0) {
+        o[j] *= c;
+        div[lo] = div[lo + 1] = o[j];
+      } else {
+        div[lo] = mad(c, o[j], div[lo]);
+        div[lo + (1 << i)] = mad(c, o[j], div[lo + (1 << i)]);
       }
     }
-    const VmsQ<A> c = vms_point(fp.v[Q], gp, mg, uv0, g, p);
-    A F[3];
-    forcing_at<Q>(pe, g, c.gphi, F);
-    rm_point(c, p.get<A>(), F, pg, vv, vgr, uv, ug, R, div);
-    return c;
   }
 };
 
@@ -286,27 +296,33 @@ k_rhs_poisson(MeshDev m, DevParams p, CoefArgs<double> cf, Ptr3 v, Ptr3 uk,
   int idx[8];
   load_corners(m, e, idx);
   const Geo<A> g = geometry<A>(m, e);
-  A pe[8];
+  constexpr double w = gauss_w<A>();
+  const PrmT<A>& k = p.get<A>();
+  const VmsElem<A> el(g, k);
   ProjFields<A> f;
-  f.load(m, idx, cf, v, uk, pk, pe);
-  const A J = g.detJ, k2 = p.get<A>().k2dt;
-  A s[8], V[3][8];
+  f.load(m, idx, cf, v, uk, pk, g, k);
+  const Forcing<A> fo(f.pe, g, k.cw);
+  const A J = g.detJ, js = -(J * k.k2dt) * A(w * w * w);
+  GradC<A> d;
   for_qp([&](auto QC) {
     constexpr int Q = decltype(QC)::value;
-    A pg[3], R[3], vv[3], div;
-    const VmsQ<A> c = f.template at<Q>(pe, g, p, pg, R, vv, div);
-    const A jr = J / c.rho, kt = k2 * c.tau;
+    A adv[3], gp[3];
+    const VmsQ<A> c = f.at(Q, el, k, adv, gp);
+    const A kt = k.k2dt * c.tau, jr = J * c.rho * A(w * w * w), jt = J * c.tau;
 #pragma unroll
-    for (int d = 0; d < 3; ++d) V[d][Q] = jr * (pg[d] - kt * R[d]);
-    s[Q] = -(J * k2 * div);
-    if (qvu)
-#pragma unroll
-      for (int i = 0; i < 3; ++i)
-        qvu[(int64_t)(Q * 3 + i) * m.n_elem + e] = (double)(J * (c.rho * vv[i] - c.tau * R[i]));
+    for (int i = 0; i < 3; ++i) {
+      const A R = f.residual(Q, i, c, adv, gp, fo, k);
+      d.sum(Q, i, c.ir * mad(-kt, R, f.gpr.at(Q, i)));
+      if (qvu)
+        qvu[(int64_t)(Q * 3 + i) * m.n_elem + e] = (double)mad(-jt, R, jr * f.vv[i][Q]);
+    }
+    f.div[Q] *= js;
   });
   A r[8];
-  interp3(s, r);
-  grad_T(V, g, r);
+  interp3<false>(f.div, r);
+  const A ca = J * A(w * w);
+  const A sc[3] = {ca * g.ih[0], ca * g.ih[1], ca * g.ih[2]};
+  d.transpose(sc, r);
   scatter<A, false>(m, idx, r, b);
 }
 
@@ -320,23 +336,25 @@ k_rhs_vu_q(MeshDev m, DevParams p, const double* __restrict__ qvu, const double*
   int idx[8];
   load_corners(m, e, idx);
   const Geo<double> g = geometry<double>(m, e);
-  QpField<double> fd;  // p_new - p_k
+  constexpr double w = gauss_w<double>();
+  GradC<double> fd;  // dt/2 J grad (p_new - p_k)
   {
     double a[8], c0[8];
     gather<double, false>(m, idx, pn, a);
     gather<double, false>(m, idx, pk, c0);
 #pragma unroll
     for (int k = 0; k < 8; ++k) a[k] -= c0[k];
-    fd.eval_grad(a);
+    const double c = w * w * g.detJ * p.d.half_dt;
+    const double cg[3] = {c * g.ih[0], c * g.ih[1], c * g.ih[2]};
+    fd.eval(a, cg);
   }
-  const double jh = g.detJ * p.d.half_dt;
-#pragma unroll 1
+  #pragma unroll
   for (int i = 0; i < 3; ++i) {
     double s[8], r[8];
 #pragma unroll
     for (int q = 0; q < 8; ++q)
-      s[q] = __ldg(qvu + (int64_t)(q * 3 + i) * m.n_elem + e) - jh * fd.grad(q, i, g);
-    interp3(s, r);
+      s[q] = (__ldg(qvu + (int64_t)(q * 3 + i) * m.n_elem + e) - fd.at(q, i)) * (w * w * w);
+    interp3<false>(s, r);
     scatter<double, true>(m, idx, r, b + i * m.n_nodes);
   }
 }
@@ -352,32 +370,39 @@ k_rhs_vu(MeshDev m, DevParams p, CoefArgs<double> cf, Ptr3 v, Ptr3 uk,
   int idx[8];
   load_corners(m, e, idx);
   const Geo<A> g = geometry<A>(m, e);
-  A pe[8];
+  constexpr double w = gauss_w<A>();
+  const PrmT<A>& k = p.get<A>();
+  const VmsElem<A> el(g, k);
   ProjFields<A> f;
-  f.load(m, idx, cf, v, uk, pk, pe);
-  QpField<A> fd;  // p_new - p_k
+  f.load(m, idx, cf, v, uk, pk, g, k);
+  const Forcing<A> fo(f.pe, g, k.cw);
+  GradC<A> fd;  // dt/2 grad (p_new - p_k)
   {
     A a[8], c0[8];
     gather<A, false>(m, idx, pn, a);
     gather<A, false>(m, idx, pk, c0);
 #pragma unroll
-    for (int k = 0; k < 8; ++k) a[k] = a[k] - c0[k];
-    fd.eval_grad(a);
+    for (int n = 0; n < 8; ++n) a[n] = a[n] - c0[n];
+    const A c = A(w * w) * k.half_dt;
+    const A cg[3] = {c * g.ih[0], c * g.ih[1], c * g.ih[2]};
+    fd.eval(a, cg);
   }
-  const A J = g.detJ, hdt = p.get<A>().half_dt;
-  A s[3][8];
+  const A j3 = g.detJ * A(w * w * w);
   for_qp([&](auto QC) {
     constexpr int Q = decltype(QC)::value;
-    A pg[3], R[3], vv[3], div;
-    const VmsQ<A> c = f.template at<Q>(pe, g, p, pg, R, vv, div);
+    A adv[3], gp[3];
+    const VmsQ<A> c = f.at(Q, el, k, adv, gp);
+    const A rw = c.rho * A(w * w * w);
 #pragma unroll
-    for (int i = 0; i < 3; ++i)
-      s[i][Q] = J * (c.rho * vv[i] - c.tau * R[i] - hdt * fd.grad(Q, i, g));
+    for (int i = 0; i < 3; ++i) {
+      const A R = f.residual(Q, i, c, adv, gp, fo, k);
+      f.vv[i][Q] = j3 * mad(rw, f.vv[i][Q], -mad(c.tau, R, fd.at(Q, i)));
+    }
   });
-#pragma unroll 1
+#pragma unroll
   for (int i = 0; i < 3; ++i) {
     A r[8];
-    interp3(s[i], r);
+    interp3<false>(f.vv[i], r);
     scatter<A, true>(m, idx, r, b + i * m.n_nodes);
   }
 }

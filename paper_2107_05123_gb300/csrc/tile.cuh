@@ -32,41 +32,13 @@
 // or 8 CTAs per SM 153 and 155 us.
 #pragma once
 
-#include "f32x2.cuh"
 #include "ops.cuh"
 #include "reduce.cuh"
 
 namespace chns {
 
-// Unnormalised 1D interpolation to the Gauss points: o0 = a + r b, o1 = r a + b with r = W1/W0;
-// each axis interpolated leaves a factor W0, which the callers fold into their constants (two
-// fused multiply-adds instead of a subtraction and two).
-// The factor is that of the rounded ratio, 1 / (1 + r), so that constants are reproduced.
-constexpr float kRf = 0.26794919243112270647f;
-constexpr double kWr = 1.0 / (1.0 + (double)kRf), kWr2 = kWr * kWr;
-
-template <class V>
-__device__ __forceinline__ void it(V a, V b, V& o0, V& o1) {
-  o0 = vfma(V(kRf), b, a);
-  o1 = vfma(V(kRf), a, b);
-}
-
-// Normalised form, o0 = a + W1 (b - a) and o1 = b - W1 (b - a): one more operation and half the
-// rounding error of a chain of six (measured 5.6e-8 against 9.7e-8 for the mass operator, whose
-// result has no differences that would drown it).
-template <class V>
-__device__ __forceinline__ void itn(V a, V b, V& o0, V& o1) {
-  const V d = b - a;
-  o0 = vfma(V((float)kW1), d, a);
-  o1 = vfma(V(-(float)kW1), d, b);
-}
-template <bool NORM, class V>
-__device__ __forceinline__ void interp(V a, V b, V& o0, V& o1) {
-  if constexpr (NORM)
-    itn(a, b, o0, o1);
-  else
-    it(a, b, o0, o1);
-}
+constexpr float kRf = (float)kRat;
+constexpr double kWr = gauss_w<F2>(), kWr2 = kWr * kWr;
 
 // Element data by columns (col = ix + 2 iy): values interpolated along z (index qz) and z
 // differences; the accumulators of the transposes are laid out the same way.
@@ -105,7 +77,7 @@ __device__ __forceinline__ void rho_qp(const V s[4][2], const PrmT<float>& k, V 
   cols_to_qp<NORM>(s, q);
 #pragma unroll
   for (int i = 0; i < 8; ++i)
-    rho[i] = vfma(V(k.alpha * (float)w), clamp_nan(q[i], 0.f, (float)(2.0 / w)), V(k.rho_m));
+    rho[i] = mad(V(k.alpha * (float)w), clamp_nan(q[i], 0.f, (float)(2.0 / w)), V(k.rho_m));
 }
 
 // Two Poisson elements from columns; A, AD: the transposes of the column values and differences.
@@ -129,7 +101,7 @@ __device__ __forceinline__ void poisson_cols(const V S[4][2], const V X[4][2], c
 #pragma unroll
       for (int y = 0; y < 2; ++y) {
         const V s = g[y][z] * (c[2 * y + 4 * z] + c[1 + 2 * y + 4 * z]);
-        if (E) ee[0] = vfma(g[y][z], s, ee[0]);
+        if (E) ee[0] = mad(g[y][z], s, ee[0]);
         g[y][z] = s;
       }
       V t0, t1;
@@ -150,15 +122,15 @@ __device__ __forceinline__ void poisson_cols(const V S[4][2], const V X[4][2], c
 #pragma unroll
       for (int x = 0; x < 2; ++x) {
         const V s = g[x][z] * (c[x + 4 * z] + c[x + 2 + 4 * z]);
-        if (E) ee[1] = vfma(g[x][z], s, ee[1]);
+        if (E) ee[1] = mad(g[x][z], s, ee[1]);
         g[x][z] = s;
       }
       V t0, t1;
       it(g[0][z], g[1][z], t0, t1);
-      A[0][z] = vfma(-sc[1], t0, A[0][z]);
-      A[2][z] = vfma(sc[1], t0, A[2][z]);
-      A[1][z] = vfma(-sc[1], t1, A[1][z]);
-      A[3][z] = vfma(sc[1], t1, A[3][z]);
+      A[0][z] = mad(-sc[1], t0, A[0][z]);
+      A[2][z] = mad(sc[1], t0, A[2][z]);
+      A[1][z] = mad(-sc[1], t1, A[1][z]);
+      A[3][z] = mad(sc[1], t1, A[3][z]);
     }
   }
   {  // z: column differences, interpolated in x and y
@@ -173,7 +145,7 @@ __device__ __forceinline__ void poisson_cols(const V S[4][2], const V X[4][2], c
 #pragma unroll
       for (int x = 0; x < 2; ++x) {
         const V s = g[x][y] * (c[x + 2 * y] + c[x + 2 * y + 4]);
-        if (E) ee[2] = vfma(g[x][y], s, ee[2]);
+        if (E) ee[2] = mad(g[x][y], s, ee[2]);
         g[x][y] = s;
       }
 #pragma unroll
@@ -181,7 +153,7 @@ __device__ __forceinline__ void poisson_cols(const V S[4][2], const V X[4][2], c
     it(t0[0], t0[1], AD[0], AD[2]);
     it(t1[0], t1[1], AD[1], AD[3]);
   }
-  if (E) *e = vfma(sc[0], ee[0], vfma(sc[1], ee[1], sc[2] * ee[2]));
+  if (E) *e = mad(sc[0], ee[0], mad(sc[1], ee[1], sc[2] * ee[2]));
 }
 
 // References of a thread's two leaves: byte offsets of their slots in 12 bits of 16. Brick pair
@@ -309,8 +281,8 @@ struct TilePoisson {
     for (int j = 0; j < 4; ++j) {
       F2 o0, o1;
       it(A[j][0], A[j][1], o0, o1);
-      r[j][0] = vfma(-sc[2], AD[j], o0);
-      r[j][1] = vfma(sc[2], AD[j], o1);
+      r[j][0] = mad(-sc[2], AD[j], o0);
+      r[j][1] = mad(sc[2], AD[j], o1);
     }
   }
 };
@@ -369,8 +341,8 @@ struct TileShift {
     cz = g.c[3];
   }
   static __device__ __forceinline__ void P(F2 a, F2 b, F2& o0, F2& o1) {
-    o0 = vfma(F2(2.f), a, b);
-    o1 = vfma(F2(2.f), b, a);
+    o0 = mad(F2(2.f), a, b);
+    o1 = mad(F2(2.f), b, a);
   }
   template <bool BR>
   __device__ __forceinline__ void apply(const PrmT<float>&, const PairRefs<BR>& pr,
@@ -393,8 +365,8 @@ struct TileShift {
       for (int x = 0; x < 2; ++x) {
         P(u[z][x], u[z + 1][x], B[z][x], B[z + 1][x]);
         const F2 dy = cy * (u[z][x] - u[z + 1][x]);
-        S[z][x] = vfma(cm, B[z][x], x ? dy - e0 : dy + e0);
-        S[z + 1][x] = vfma(cm, B[z + 1][x], -(x ? dy + e1 : dy - e1));
+        S[z][x] = mad(cm, B[z][x], x ? dy - e0 : dy + e0);
+        S[z + 1][x] = mad(cm, B[z + 1][x], -(x ? dy + e1 : dy - e1));
       }
     }
 #pragma unroll
