@@ -20,7 +20,6 @@
 namespace chns {
 
 constexpr int kVecThreads = 256;
-constexpr int kMdBlocks = 256;  // blocks per multi-dot row (partials: rows x kMdBlocks)
 
 // device scalar slots (offsets from ws.red + kScalarBase)
 enum Slot { S_RZ0 = 0, S_RZ1 = 1, S_PQ = 2, S_RR = 3, S_TMP = 8, S_AUX = 16, S_MD = 64 };
@@ -367,6 +366,139 @@ void orth_update(const T* V, int64_t ld, int nk, const double* h, T* w, int64_t 
                  cudaStream_t s) {
   note_launch();
   k_orth_update_scale<T, NORMALISE><<<grid, kVecThreads, 0, s>>>(V, ld, nk, h, w, n);
+}
+
+// One Gram-Schmidt step of GMRES in one cooperative launch (all CTAs resident: they wait on one
+// another at a grid barrier): h = V^T w and w.w, w -= V h, and when the new vector lost more than
+// half its norm to the projection a second pass, then w normalised. out[k] = the column of the
+// Hessenberg matrix (k < nk), out[nk] = the norm of the new vector before it was normalised.
+// Each CTA keeps its slice of w in shared memory. Sums over the CTAs are FP64 atomics into acc
+// (two rows of kArnoldiMax, zero on entry; acc_next is cleared for the next step). Against the
+// separate kernels (multi-dot, final sum, update, each twice, and a host decision between them) it
+// saves five launches and a synchronisation per GMRES iteration, which is what a basis that fits
+// the L2 costs: its time is latency, about 10 us for 30 vectors of 36,530.
+constexpr int kArnoldiThreads = 512;
+constexpr int kArnoldiMax = 64;          // restart + 1 sums
+constexpr int kArnoldiSlice = 40 * 1024;  // bytes of w per CTA: longer vectors take the kernels below
+
+// Waits until all CTAs of the launch have arrived `round` times; false when it gave up (a limit of
+// about a second: nothing the caller can continue from).
+__device__ __forceinline__ bool grid_arrive_wait(unsigned* bar, unsigned round) {
+  __shared__ int ok;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    atomicAdd(bar, 1u);
+    const unsigned want = round * gridDim.x;
+    int spins = 0;
+    while (*(volatile unsigned*)bar < want && spins < (1 << 22)) ++spins;
+    __threadfence();
+    ok = spins < (1 << 22);
+  }
+  __syncthreads();
+  return ok;
+}
+
+// acc[k] += sum over the slice of V_k w (k < nk) and w.w (k = nk): one warp per row, four rows at a
+// time so that their loads overlap
+template <class T>
+__device__ __forceinline__ void slice_dots(const T* __restrict__ V, int64_t ld, int nk,
+                                           const T* ws, int64_t i0, int len, double* acc) {
+  constexpr int W = kArnoldiThreads / 32, R = 2;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int k0 = warp; k0 <= nk; k0 += R * W) {
+    typename Acc<T>::type a[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) a[r] = Acc<T>::zero();
+#pragma unroll 4
+    for (int i = lane; i < len; i += 32) {
+      const T wi = ws[i];
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const int k = k0 + r * W;
+        if (k < nk) Acc<T>::fma(a[r], V[(int64_t)k * ld + i0 + i], wi);
+        if (k == nk) Acc<T>::fma(a[r], wi, wi);
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const int k = k0 + r * W;
+      if (k > nk) continue;
+      const auto t = warp_sum(a[r]);
+      if (lane == 0) atomicAdd(acc + k, acc_value(t));
+    }
+  }
+}
+
+// ws -= V h over the slice, in the vector type
+template <class T>
+__device__ __forceinline__ void slice_update(const T* __restrict__ V, int64_t ld, int nk,
+                                             const T* hs, T* ws, int64_t i0, int len) {
+  for (int i = threadIdx.x; i < len; i += kArnoldiThreads) {
+    T v = ws[i];
+#pragma unroll 8
+    for (int k = 0; k < nk; ++k) v -= hs[k] * V[(int64_t)k * ld + i0 + i];
+    ws[i] = v;
+  }
+}
+
+template <class T>
+__global__ void __launch_bounds__(kArnoldiThreads)
+k_arnoldi(const T* __restrict__ V, int64_t ld, int nk, T* __restrict__ w, int64_t n, int chunk,
+          double* __restrict__ acc, double* __restrict__ acc_next, unsigned* __restrict__ bar,
+          unsigned* __restrict__ bar_next, double* __restrict__ out) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  T* ws = reinterpret_cast<T*>(smem_raw);
+  __shared__ T hs[kArnoldiMax];
+  __shared__ double hd[kArnoldiMax];
+  __shared__ double s_nn;
+  const int64_t i0 = (int64_t)blockIdx.x * chunk;
+  const int len = (int)(i0 >= n ? 0 : (n - i0 < chunk ? n - i0 : chunk));
+  for (int i = threadIdx.x; i < len; i += kArnoldiThreads) ws[i] = w[i0 + i];
+  __syncthreads();
+  slice_dots(V, ld, nk, ws, i0, len, acc);
+  unsigned round = 1;
+  bool ok = grid_arrive_wait(bar, round);
+  if (blockIdx.x == 0) {
+    for (int k = threadIdx.x; k < 2 * kArnoldiMax; k += kArnoldiThreads) acc_next[k] = 0.0;
+    if (threadIdx.x == 0) *bar_next = 0u;
+  }
+  // coefficients, |w|^2 - |h|^2 (Pythagoras); every CTA forms the same values
+  auto read = [&](const double* a) {
+    if (threadIdx.x < nk) {
+      const double v = ((volatile const double*)a)[threadIdx.x];
+      hd[threadIdx.x] = v;
+      hs[threadIdx.x] = (T)v;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      double hh = 0.0;
+      for (int k = 0; k < nk; ++k) hh += hd[k] * hd[k];
+      s_nn = ((volatile const double*)a)[nk] - hh;
+    }
+    __syncthreads();
+  };
+  read(acc);
+  double nn = s_nn;
+  const double ww = ((volatile const double*)acc)[nk];
+  double h1 = threadIdx.x < nk ? hd[threadIdx.x] : 0.0;
+  slice_update(V, ld, nk, hs, ws, i0, len);
+  if (!(nn > 0.5 * ww) && ok) {
+    __syncthreads();
+    slice_dots(V, ld, nk, ws, i0, len, acc + kArnoldiMax);
+    ok = grid_arrive_wait(bar, ++round);
+    read(acc + kArnoldiMax);
+    nn = s_nn;
+    if (threadIdx.x < nk) h1 += hd[threadIdx.x];
+    slice_update(V, ld, nk, hs, ws, i0, len);
+  }
+  const T sc = (T)(nn > 0.0 ? rsqrt(nn) : 1.0);
+  for (int i = threadIdx.x; i < len; i += kArnoldiThreads) w[i0 + i] = ws[i] * sc;
+  if (blockIdx.x == 0) {
+    if (threadIdx.x < nk) out[threadIdx.x] = h1;
+    // a NaN norm stops the solve (as does a barrier that gave up)
+    if (threadIdx.x == 0) out[nk] = !ok ? nan("") : nn > 0.0 ? sqrt(nn) : nn == nn ? 0.0 : nn;
+  }
 }
 
 template <class T>
@@ -1033,8 +1165,40 @@ unsigned multidot(const chns_mesh* m, const T* V, int64_t ld, int nk, const T* w
   return chunks;
 }
 
+// scratch of k_arnoldi in the reduction partials: sums [2 parities][2][kArnoldiMax], results
+// [2][kArnoldiMax], barriers [2]
+constexpr int kArnoldiPinned = 128;  // offset in the pinned scalars
+constexpr size_t kArnoldiBytes = (6 * kArnoldiMax + 2) * sizeof(double);
+static_assert(6 * kArnoldiMax + 2 <= kRedSlots && CHNS_GMRES_MAX_RESTART + 1 <= kArnoldiMax &&
+                  kArnoldiPinned + 2 * kArnoldiMax <= 1024,
+              "k_arnoldi scratch");
+static double* arnoldi_acc(const Ctx& c, int par) {
+  return c.m->ws.red + 2 * kRedSlots + par * 2 * kArnoldiMax;
+}
+static double* arnoldi_out(const Ctx& c, int par) {
+  return c.m->ws.red + 2 * kRedSlots + (4 + par) * kArnoldiMax;
+}
+
+template <class T>
+chns_status arnoldi(const Ctx& c, const T* V, int64_t ld, int nk, T* w, int64_t n, int chunk,
+                    int par) {
+  unsigned* bar = reinterpret_cast<unsigned*>(arnoldi_acc(c, 0) + 6 * kArnoldiMax);
+  double *acc = arnoldi_acc(c, par), *next = arnoldi_acc(c, par ^ 1), *out = arnoldi_out(c, par);
+  unsigned *b0 = bar + 2 * par, *b1 = bar + 2 * (par ^ 1);
+  void* args[] = {(void*)&V, (void*)&ld, (void*)&nk,   (void*)&w,  (void*)&n, (void*)&chunk,
+                  (void*)&acc, (void*)&next, (void*)&b0, (void*)&b1, (void*)&out};
+  note_launch();
+  CHNS_CUDA(cudaLaunchCooperativeKernel((const void*)k_arnoldi<T>, dim3((unsigned)c.m->sm_count),
+                                        dim3(kArnoldiThreads), args, (size_t)chunk * sizeof(T),
+                                        c.s));
+  return CHNS_OK;
+}
+
 // Right-preconditioned restarted GMRES with classical Gram-Schmidt and one re-orthogonalisation
-// pass; the second pass also returns w.w so that the new norm needs no extra reduction.
+// pass; the second pass also returns w.w so that the new norm needs no extra reduction. Where the
+// vectors are short (k_arnoldi) the Gram-Schmidt step is one launch and, unless the preconditioner
+// is expensive (spc), the host looks at column j while the kernels of column j + 1 run: the solve
+// may do the kernels of one column more than it uses.
 template <class T>
 chns_status gmres(const Ctx& c, const T* b, T* x, const T* dinv, bool block2, double tol_abs,
                   int max_it, int restart, T* V, T* z, int* iters, double* rnorm,
@@ -1044,13 +1208,26 @@ chns_status gmres(const Ctx& c, const T* b, T* x, const T* dinv, bool block2, do
   // vectors in the same buffer, and the update is x += Z y
   T* Zb = V + (int64_t)(restart + 1) * ld;
   const unsigned vg = vgrid(c.m, n);
-  const unsigned mdb = (unsigned)std::max<int64_t>(1, std::min<int64_t>(kMdBlocks, (n + 255) / 256));
   double* hdev = c.S + S_MD;
   std::vector<double> H((size_t)(restart + 1) * restart, 0.0), cs(restart), sn(restart),
       g(restart + 1), y(restart), h(restart + 2);
   int it = 0;
   double beta = 0.0;
   chns_status st;
+  // slices of k_arnoldi: one CTA per SM
+  const int64_t chunk = (n + c.m->sm_count - 1) / std::max(c.m->sm_count, 1);
+  const bool fused = chunk * (int64_t)sizeof(T) <= kArnoldiSlice;
+  struct Events {
+    cudaEvent_t e[2] = {nullptr, nullptr};
+    ~Events() {
+      for (auto x : e)
+        if (x) cudaEventDestroy(x);
+    }
+  } ev;
+  if (fused) {
+    for (auto& x : ev.e) CHNS_CUDA(cudaEventCreateWithFlags(&x, cudaEventDisableTiming));
+    CHNS_CUDA(cudaMemsetAsync(arnoldi_acc(c, 0), 0, kArnoldiBytes, c.s));
+  }
   auto Hij = [&](int i, int j) -> double& { return H[(size_t)i * restart + j]; };
   for (;;) {
     // r = b - A x into V_0
@@ -1073,7 +1250,42 @@ chns_status gmres(const Ctx& c, const T* b, T* x, const T* dinv, bool block2, do
     std::fill(g.begin(), g.end(), 0.0);
     g[0] = beta;
     int jend = 0;
-    for (int j = 0; j < restart; ++j) {
+    bool stop = false;
+    // Givens rotations of column j (H and hn = its subdiagonal entry); stop: converged or the end
+    auto column = [&](int j, double hn) -> chns_status {
+      Hij(j + 1, j) = hn;
+      if (!std::isfinite(hn)) {
+        set_error("krylov: NaN/Inf in GMRES");
+        *iters = it;
+        *rnorm = hn;
+        return CHNS_ENAN;
+      }
+      for (int i = 0; i < j; ++i) {
+        double t = cs[i] * Hij(i, j) + sn[i] * Hij(i + 1, j);
+        Hij(i + 1, j) = -sn[i] * Hij(i, j) + cs[i] * Hij(i + 1, j);
+        Hij(i, j) = t;
+      }
+      double a = Hij(j, j), bb = Hij(j + 1, j);
+      double rden = std::hypot(a, bb);
+      cs[j] = rden > 0.0 ? a / rden : 1.0;
+      sn[j] = rden > 0.0 ? bb / rden : 0.0;
+      Hij(j, j) = rden;
+      Hij(j + 1, j) = 0.0;
+      g[j + 1] = -sn[j] * g[j];
+      g[j] = cs[j] * g[j];
+      ++it;
+      jend = j + 1;
+      stop = std::fabs(g[j + 1]) <= tol_abs || it >= max_it || hn == 0.0;
+      return CHNS_OK;
+    };
+    // the column that k_arnoldi left in the pinned slot of parity j & 1
+    auto fused_column = [&](int j) -> chns_status {
+      CHNS_CUDA(cudaEventSynchronize(ev.e[j & 1]));
+      const volatile double* o = c.m->ws.h_pinned + kArnoldiPinned + (j & 1) * kArnoldiMax;
+      for (int i = 0; i <= j; ++i) Hij(i, j) = o[i];
+      return column(j, o[j + 1]);
+    };
+    for (int j = 0; j < restart && !stop; ++j) {
       T* vj = V + (int64_t)j * ld;
       T* w = V + (int64_t)(j + 1) * ld;
       T* zj = spc ? Zb + (int64_t)j * ld : z;
@@ -1089,9 +1301,25 @@ chns_status gmres(const Ctx& c, const T* b, T* x, const T* dinv, bool block2, do
       }
       st = apply_T<T>(c, zj, w);
       if (st != CHNS_OK) return st;
+      const int nk = j + 1;
+      if (fused) {
+        st = arnoldi<T>(c, V, ld, nk, w, n, (int)chunk, j & 1);
+        if (st != CHNS_OK) return st;
+        CHNS_CUDA(cudaMemcpyAsync(c.m->ws.h_pinned + kArnoldiPinned + (j & 1) * kArnoldiMax,
+                                  arnoldi_out(c, j & 1), (nk + 1) * sizeof(double),
+                                  cudaMemcpyDeviceToHost, c.s));
+        CHNS_CUDA(cudaEventRecord(ev.e[j & 1], c.s));
+        if (spc) {
+          st = fused_column(j);
+        } else {
+          if (j > 0) st = fused_column(j - 1);
+          if (st == CHNS_OK && !stop && j + 1 == restart) st = fused_column(j);
+        }
+        if (st != CHNS_OK) return st;
+        continue;
+      }
       // classical Gram-Schmidt: h = V^T w and w.w in one pass; a second pass only when the
       // new vector lost more than half its norm to the projection (cancellation)
-      int nk = j + 1;
       const unsigned md2 = multidot(c.m, V, ld, nk, w, n, c.m->ws.md_part, c.s);
       note_launch();
       k_multidot_final<<<nk + 1, kVecThreads, 0, c.s>>>(c.m->ws.md_part, (int)md2, hdev);
@@ -1121,34 +1349,10 @@ chns_status gmres(const Ctx& c, const T* b, T* x, const T* dinv, bool block2, do
         }
         hn2 = h[nk] - h2;
       }
-      const double hn = std::sqrt(std::max(0.0, hn2));
-      Hij(j + 1, j) = hn;
-      if (!std::isfinite(hn)) {
-        set_error("krylov: NaN/Inf in GMRES");
-        *iters = it;
-        *rnorm = hn;
-        return CHNS_ENAN;
-      }
-      if (hn > 0.0) {
-        orth_update<T, true>(V, ld, nk, hdev, w, n, vg, c.s);
-      }
-      // Givens rotations
-      for (int i = 0; i < j; ++i) {
-        double t = cs[i] * Hij(i, j) + sn[i] * Hij(i + 1, j);
-        Hij(i + 1, j) = -sn[i] * Hij(i, j) + cs[i] * Hij(i + 1, j);
-        Hij(i, j) = t;
-      }
-      double a = Hij(j, j), bb = Hij(j + 1, j);
-      double rden = std::hypot(a, bb);
-      cs[j] = rden > 0.0 ? a / rden : 1.0;
-      sn[j] = rden > 0.0 ? bb / rden : 0.0;
-      Hij(j, j) = rden;
-      Hij(j + 1, j) = 0.0;
-      g[j + 1] = -sn[j] * g[j];
-      g[j] = cs[j] * g[j];
-      ++it;
-      jend = j + 1;
-      if (std::fabs(g[j + 1]) <= tol_abs || it >= max_it || hn == 0.0) break;
+      const double hn = hn2 > 0.0 ? std::sqrt(hn2) : hn2 == hn2 ? 0.0 : hn2;
+      if (hn > 0.0) orth_update<T, true>(V, ld, nk, hdev, w, n, vg, c.s);
+      st = column(j, hn);
+      if (st != CHNS_OK) return st;
     }
     // back substitution and update x += M^-1 V y
     for (int i = jend - 1; i >= 0; --i) {
