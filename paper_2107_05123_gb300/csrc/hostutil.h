@@ -36,19 +36,29 @@ inline uint64_t morton(uint64_t x, uint64_t y, uint64_t z) {
   return spread3(x) | (spread3(y) << 1) | (spread3(z) << 2);
 }
 
-// Run f(begin, end) over [0, n) on up to hw threads.
+// Threads for a loop over n items, and f(part, begin, end) over [0, n) cut into that many parts.
+inline int threads_for(int64_t n) {
+  const int nt = (int)std::max(1u, std::min(16u, std::thread::hardware_concurrency()));
+  return (int)std::max<int64_t>(1, std::min<int64_t>(nt, n / 4096));
+}
 template <class F>
-void parallel_for(int64_t n, F f) {
-  int nt = (int)std::max(1u, std::min(16u, std::thread::hardware_concurrency()));
-  if (n < 65536) nt = 1;
+void parallel_parts(int64_t n, int nt, F f) {
   std::vector<std::thread> th;
-  int64_t chunk = (n + nt - 1) / nt;
+  const int64_t chunk = (n + nt - 1) / nt;
   for (int t = 0; t < nt; ++t) {
-    int64_t b = t * chunk, e = std::min(n, b + chunk);
+    const int64_t b = t * chunk, e = std::min(n, b + chunk);
     if (b >= e) break;
-    th.emplace_back([=]() { f(b, e); });
+    if (e == n)
+      f(t, b, e);
+    else
+      th.emplace_back([=, &f]() { f(t, b, e); });
   }
   for (auto& t : th) t.join();
+}
+// Run f(begin, end) over [0, n) on up to 16 threads.
+template <class F>
+void parallel_for(int64_t n, F f) {
+  parallel_parts(n, threads_for(n), [&](int, int64_t b, int64_t e) { f(b, e); });
 }
 
 }  // namespace host

@@ -67,6 +67,7 @@ struct MeshDev {
 };
 
 struct Workspace {
+  void* slab = nullptr;  // holds every device array below
   // FP64 vectors (sized for 3 components) and FP32 mirrors
   std::vector<double*> v64;
   std::vector<float*> v32;

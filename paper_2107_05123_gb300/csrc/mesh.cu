@@ -14,6 +14,7 @@
 #include <atomic>
 #include <cmath>
 #include <cstring>
+#include <iterator>
 #include <memory>
 #include <numeric>
 #include <thread>
@@ -28,13 +29,6 @@ using host::compact3;
 using host::kFull;
 using host::morton;
 using host::parallel_for;
-
-struct Cancel {
-  uint64_t key;      // Morton key of the midpoint/centre
-  int32_t leaf;
-  int32_t kind;      // 0..11 edges, 12..17 faces
-  bool operator<(const Cancel& o) const { return key < o.key; }
-};
 
 // Corner c (0..7, bits x,y,z) of a leaf.
 inline void corner_xyz(const uint32_t* a, uint64_t s, int c, uint64_t out[3]) {
@@ -88,23 +82,44 @@ static chns_status alloc_workspace(chns_mesh* m, bool light) {
     CHNS_CUDA(cudaStreamCreateWithFlags(&m->cap_stream, cudaStreamNonBlocking));
     return CHNS_OK;
   }
+  // one allocation, cut into 256-byte aligned arrays (some forty cudaMalloc calls took longer than
+  // the tables of a small mesh)
   w.v64.assign(kNumVec64, nullptr);
   w.v32.assign(kNumVec32, nullptr);
-  for (auto& p : w.v64) CHNS_CUDA(cudaMalloc(&p, n3 * sizeof(double)));
-  for (auto& p : w.v32) CHNS_CUDA(cudaMalloc(&p, n3 * sizeof(float)));
-  CHNS_CUDA(cudaMalloc(&w.gm_V, (size_t)(CHNS_GMRES_MAX_RESTART + 1) * n3 * sizeof(double)));
-  CHNS_CUDA(cudaMalloc(&w.gm_V32, (size_t)(CHNS_GMRES_MAX_RESTART + 1) * n3 * sizeof(float)));
-  CHNS_CUDA(cudaMalloc(&w.red, (size_t)(kScalarBase + 1024) * sizeof(double)));
+  struct Part {
+    void** p;
+    size_t bytes;
+  };
+  std::vector<Part> parts;
+  auto part = [&](auto*& p, size_t count) {
+    parts.push_back({(void**)&p, (count * sizeof(*p) + 255) / 256 * 256});
+  };
+  for (auto& p : w.v64) part(p, n3);
+  for (auto& p : w.v32) part(p, n3);
+  part(w.gm_V, (size_t)(CHNS_GMRES_MAX_RESTART + 1) * n3);
+  part(w.gm_V32, (size_t)(CHNS_GMRES_MAX_RESTART + 1) * n3);
+  part(w.red, (size_t)(kScalarBase + 1024));
+  part(w.counter, 64);
+  float* c32 = nullptr;
+  __nv_bfloat16* c16 = nullptr;
+  part(c32, (size_t)10 * N);
+  part(c16, (size_t)8 * N);
+  part(w.coef64, (size_t)16 * N);
+  part(w.part_big, (size_t)(m->d.n_elem / 64 + 64));
+  part(w.md_part, (size_t)(CHNS_GMRES_MAX_RESTART + 2) * kMdMaxBlocks);
+  size_t total = 0;
+  for (auto& q : parts) total += q.bytes;
+  CHNS_CUDA(cudaMalloc(&w.slab, total));
+  char* at = static_cast<char*>(w.slab);
+  for (auto& q : parts) {
+    *q.p = at;
+    at += q.bytes;
+  }
+  w.coef32 = c32;
+  w.coef16 = c16;
   CHNS_CUDA(cudaMemset(w.red, 0, (size_t)(kScalarBase + 1024) * sizeof(double)));
-  CHNS_CUDA(cudaMalloc(&w.counter, 64 * sizeof(unsigned int)));
   CHNS_CUDA(cudaMemset(w.counter, 0, 64 * sizeof(unsigned int)));
   CHNS_CUDA(cudaMallocHost(&w.h_pinned, 1024 * sizeof(double)));
-  CHNS_CUDA(cudaMalloc(&w.coef32, (size_t)10 * N * sizeof(float)));
-  CHNS_CUDA(cudaMalloc(&w.coef16, (size_t)8 * N * sizeof(__nv_bfloat16)));
-  CHNS_CUDA(cudaMalloc(&w.coef64, (size_t)16 * N * sizeof(double)));
-  CHNS_CUDA(cudaMalloc(&w.part_big, (size_t)(m->d.n_elem / 64 + 64) * sizeof(double)));
-  CHNS_CUDA(cudaMalloc(&w.md_part,
-                       (size_t)(CHNS_GMRES_MAX_RESTART + 2) * kMdMaxBlocks * sizeof(double)));
   CHNS_CUDA(cudaStreamCreateWithFlags(&m->cap_stream, cudaStreamNonBlocking));
   return CHNS_OK;
 }
@@ -127,18 +142,8 @@ void free_mesh(chns_mesh* m) {
   dfree(m->d_geo);
   dfree(m->d_node_int);
   Workspace& w = m->ws;
-  for (auto p : w.v64) dfree(p);
-  for (auto p : w.v32) dfree(p);
-  dfree(w.gm_V);
-  dfree(w.gm_V32);
-  dfree(w.red);
-  dfree(w.counter);
+  dfree(w.slab);
   if (w.h_pinned) cudaFreeHost(w.h_pinned);
-  dfree(w.coef32);
-  dfree(w.coef16);
-  dfree(w.coef64);
-  dfree(w.part_big);
-  dfree(w.md_part);
   dfree(m->mq.qd64);
   dfree(m->mq.qd32);
   for (int p = 0; p < 2; ++p)
@@ -493,50 +498,78 @@ chns_status build_mesh(const uint32_t* anchors, const uint8_t* levels, int64_t n
   });
   CHNS_CHECK(!unbalanced.load(), CHNS_EUNBALANCED, "leaves are not 2:1 balanced");
 
-  // ---- unique corner points
+  // ---- unique corner points: the leaves' anchors (distinct and sorted already) and the corners that
+  // are no leaf's anchor (on upper domain faces, and where a coarser leaf lies beyond), which alone
+  // are sorted
   std::vector<uint64_t> ckey((size_t)n * 8);
-  parallel_for(n, [&](int64_t b, int64_t e) {
-    for (int64_t i = b; i < e; ++i) {
-      uint64_t s = kFull >> levels[i];
-      for (int c = 0; c < 8; ++c) {
-        uint64_t q[3];
-        corner_xyz(anchors + 3 * i, s, c, q);
-        ckey[8 * i + c] = morton(q[0], q[1], q[2]);
+  std::vector<uint64_t> pts;
+  {
+    const int nt = host::threads_for(n);
+    std::vector<std::vector<uint64_t>> extra(nt);
+    std::atomic<bool> failed(false);
+    host::parallel_parts(n, nt, [&](int t, int64_t b, int64_t e) {
+     try {
+      for (int64_t i = b; i < e; ++i) {
+        uint64_t s = kFull >> levels[i];
+        for (int c = 0; c < 8; ++c) {
+          uint64_t q[3];
+          corner_xyz(anchors + 3 * i, s, c, q);
+          const uint64_t k = morton(q[0], q[1], q[2]);
+          ckey[8 * i + c] = k;
+          if (c == 0) continue;
+          // the next leaves in Morton order hold most of the anchors
+          bool found = false;
+          for (int64_t j = i + 1; j < std::min(i + 8, n) && !found; ++j) found = lkey[j] == k;
+          if (!found && !std::binary_search(lkey.begin(), lkey.end(), k)) extra[t].push_back(k);
+        }
       }
+      std::sort(extra[t].begin(), extra[t].end());
+      extra[t].erase(std::unique(extra[t].begin(), extra[t].end()), extra[t].end());
+     } catch (const std::bad_alloc&) {  // no exception leaves a thread
+       failed.store(true);
+     }
+    });
+    if (failed.load()) throw std::bad_alloc();
+    std::vector<uint64_t> all;
+    for (auto& v : extra) {
+      std::vector<uint64_t> m;
+      m.reserve(all.size() + v.size());
+      std::set_union(all.begin(), all.end(), v.begin(), v.end(), std::back_inserter(m));
+      all.swap(m);
     }
-  });
-  std::vector<uint64_t> pts(ckey);
-  std::sort(pts.begin(), pts.end());
-  pts.erase(std::unique(pts.begin(), pts.end()), pts.end());
+    pts.resize((size_t)n + all.size());
+    std::merge(lkey.begin(), lkey.end(), all.begin(), all.end(), pts.begin());
+  }
   const int64_t NP = (int64_t)pts.size();
 
-  // ---- cancellation positions and hanging detection
-  std::vector<Cancel> canc((size_t)n * 18);
+  // ---- hanging detection: a corner point at a cancellation position of some leaf (18 leaf + kind;
+  // several leaves may report a point, all with the same parents). Leaves of the finest level have
+  // nothing inside their edges and faces.
+  std::vector<std::atomic<int64_t>> hang_src((size_t)NP);
+  parallel_for(NP, [&](int64_t b, int64_t e) {
+    for (int64_t p = b; p < e; ++p) hang_src[p].store(-1, std::memory_order_relaxed);
+  });
   parallel_for(n, [&](int64_t b, int64_t e) {
     for (int64_t i = b; i < e; ++i) {
+      if (levels[i] == maxl) continue;
       uint64_t s = kFull >> levels[i], h = s / 2;
       for (int k = 0; k < 18; ++k) {
         int par[4], mh[3], bb[3];
         cancel_geom(k, par, mh, bb);
         uint64_t q[3];
         for (int d = 0; d < 3; ++d) q[d] = anchors[3 * i + d] + bb[d] * s + mh[d] * h;
-        canc[18 * i + k] = Cancel{morton(q[0], q[1], q[2]), (int32_t)i, (int32_t)k};
+        const uint64_t key = morton(q[0], q[1], q[2]);
+        auto it = std::lower_bound(pts.begin(), pts.end(), key);
+        if (it != pts.end() && *it == key)
+          hang_src[it - pts.begin()].store(18 * i + k, std::memory_order_relaxed);
       }
-    }
-  });
-  std::sort(canc.begin(), canc.end());
-  std::vector<int32_t> hang_src(NP, -1);   // index into canc of a cancellation at this point
-  parallel_for(NP, [&](int64_t b, int64_t e) {
-    for (int64_t p = b; p < e; ++p) {
-      auto it = std::lower_bound(canc.begin(), canc.end(), Cancel{pts[p], 0, 0});
-      if (it != canc.end() && it->key == pts[p]) hang_src[p] = int32_t(it - canc.begin());
     }
   });
 
   // ---- numbering: independent nodes in Morton order (pts is sorted by Morton key)
   std::vector<int64_t> pid(NP);
   int64_t N = 0, H = 0;
-  for (int64_t p = 0; p < NP; ++p) pid[p] = hang_src[p] < 0 ? N++ : -(++H);
+  for (int64_t p = 0; p < NP; ++p) pid[p] = hang_src[p].load(std::memory_order_relaxed) < 0 ? N++ : -(++H);
   CHNS_CHECK(N < (int64_t(1) << 29) && H < (int64_t(1) << 29), CHNS_EINVAL, "mesh too large");
 
   auto point_index = [&](uint64_t key) -> int64_t {
@@ -547,46 +580,50 @@ chns_status build_mesh(const uint32_t* anchors, const uint8_t* levels, int64_t n
 
   m->node_coords.resize((size_t)3 * N);
   m->node_bnd.resize((size_t)N);
+  parallel_for(NP, [&](int64_t b0, int64_t e0) {
+    for (int64_t p = b0; p < e0; ++p) {
+      if (pid[p] < 0) continue;
+      uint64_t x = compact3(pts[p]), y = compact3(pts[p] >> 1), z = compact3(pts[p] >> 2);
+      int64_t j = pid[p];
+      m->node_coords[3 * j] = (uint32_t)x;
+      m->node_coords[3 * j + 1] = (uint32_t)y;
+      m->node_coords[3 * j + 2] = (uint32_t)z;
+      bool b = x == 0 || y == 0 || z == 0 || x == kFull || y == kFull || z == kFull;
+      m->node_bnd[j] = b ? 1 : 0;
+    }
+  });
   int64_t nb = 0;
-  for (int64_t p = 0; p < NP; ++p) {
-    if (pid[p] < 0) continue;
-    uint64_t x = compact3(pts[p]), y = compact3(pts[p] >> 1), z = compact3(pts[p] >> 2);
-    int64_t j = pid[p];
-    m->node_coords[3 * j] = (uint32_t)x;
-    m->node_coords[3 * j + 1] = (uint32_t)y;
-    m->node_coords[3 * j + 2] = (uint32_t)z;
-    bool b = x == 0 || y == 0 || z == 0 || x == kFull || y == kFull || z == kFull;
-    m->node_bnd[j] = b ? 1 : 0;
-    nb += b;
-  }
+  for (uint8_t v : m->node_bnd) nb += v;
   auto flagged = [&](int64_t j) -> int32_t {
     return (int32_t)j | (m->node_bnd[j] ? kDirBit : 0);
   };
 
   // hanging table
   std::vector<int4> hang((size_t)std::max<int64_t>(H, 1));
-  bool bad = false;
-  for (int64_t p = 0; p < NP; ++p) {
-    if (pid[p] >= 0) continue;
-    int64_t h = -pid[p] - 1;
-    const Cancel& c = canc[hang_src[p]];
-    int par[4], mh[3], bb[3];
-    int np = cancel_geom(c.kind, par, mh, bb);
-    uint64_t s = kFull >> levels[c.leaf];
-    int32_t out[4] = {-1, -1, -1, -1};
-    for (int k = 0; k < np; ++k) {
-      uint64_t q[3];
-      corner_xyz(anchors + 3 * c.leaf, s, par[k], q);
-      int64_t pp = point_index(morton(q[0], q[1], q[2]));
-      if (pp < 0 || pid[pp] < 0) {
-        bad = true;
-        break;
+  std::atomic<bool> bad(false);
+  parallel_for(NP, [&](int64_t b, int64_t e) {
+    for (int64_t p = b; p < e; ++p) {
+      if (pid[p] >= 0) continue;
+      int64_t h = -pid[p] - 1;
+      const int64_t src = hang_src[p].load(std::memory_order_relaxed), leaf = src / 18;
+      int par[4], mh[3], bb[3];
+      int np = cancel_geom((int)(src % 18), par, mh, bb);
+      uint64_t s = kFull >> levels[leaf];
+      int32_t out[4] = {-1, -1, -1, -1};
+      for (int k = 0; k < np; ++k) {
+        uint64_t q[3];
+        corner_xyz(anchors + 3 * leaf, s, par[k], q);
+        int64_t pp = point_index(morton(q[0], q[1], q[2]));
+        if (pp < 0 || pid[pp] < 0) {
+          bad.store(true);
+          break;
+        }
+        out[k] = flagged(pid[pp]);
       }
-      out[k] = flagged(pid[pp]);
+      hang[h] = make_int4(out[0], out[1], out[2], out[3]);
     }
-    hang[h] = make_int4(out[0], out[1], out[2], out[3]);
-  }
-  CHNS_CHECK(!bad, CHNS_EUNBALANCED, "hanging node whose parent is not an independent node");
+  });
+  CHNS_CHECK(!bad.load(), CHNS_EUNBALANCED, "hanging node whose parent is not an independent node");
 
   // element corner table
   std::vector<int32_t> enode((size_t)n * 8);

@@ -159,8 +159,17 @@ void balance_and_emit(std::vector<std::vector<uint64_t>>& split, int lmax,
             for (int64_t x = lo[0]; x <= hi[0]; ++x) req[8 * i + k++] = host::morton(x, y, z);
       }
     });
+    // neighbours in Morton order mostly ask for the same parents: keep one of each run before the
+    // sort
+    size_t kept = 0;
+    for (size_t i = 0; i < req.size(); ++i) {
+      const uint64_t r = req[i];
+      bool seen = r == UINT64_MAX;
+      for (size_t j = kept > 8 ? kept - 8 : 0; j < kept && !seen; ++j) seen = req[j] == r;
+      if (!seen) req[kept++] = r;
+    }
+    req.resize(kept);
     sort_unique(req);
-    if (!req.empty() && req.back() == UINT64_MAX) req.pop_back();
     split[l - 1].insert(split[l - 1].end(), req.begin(), req.end());
   }
   if (lmax >= 1) sort_unique(split[0]);
@@ -173,6 +182,7 @@ void balance_and_emit(std::vector<std::vector<uint64_t>>& split, int lmax,
   for (int l = 0; l < lmax; ++l) {
     const std::vector<uint64_t>& S = split[l];
     const std::vector<uint64_t>* nxt = l + 1 < lmax ? &split[l + 1] : nullptr;
+    const size_t first = leaves.size();  // the level's leaves come in Morton order
     for (uint64_t s : S) {
       const uint64_t cx = host::compact3(s), cy = host::compact3(s >> 1), cz = host::compact3(s >> 2);
       for (int ch = 0; ch < 8; ++ch) {
@@ -184,8 +194,8 @@ void balance_and_emit(std::vector<std::vector<uint64_t>>& split, int lmax,
         leaves.emplace_back(host::morton(kx << sh, ky << sh, kz << sh), (uint8_t)(l + 1));
       }
     }
+    std::inplace_merge(leaves.begin(), leaves.begin() + (ptrdiff_t)first, leaves.end());
   }
-  std::sort(leaves.begin(), leaves.end());
   A.resize(3 * leaves.size());
   L.resize(leaves.size());
   for (size_t i = 0; i < leaves.size(); ++i) {
@@ -211,7 +221,10 @@ chns_status new_leaves(const chns_mesh* m, const int8_t* fl, std::vector<uint32_
   std::vector<std::vector<uint64_t>> split(CHNS_MAXD);
   int lmax = 0;
   auto add_leaf = [&](const uint32_t* a, int l) {
-    if (l >= 1) split[l - 1].push_back(okey(a, l - 1));
+    if (l >= 1) {  // siblings follow one another
+      const uint64_t k = okey(a, l - 1);
+      if (split[l - 1].empty() || split[l - 1].back() != k) split[l - 1].push_back(k);
+    }
     lmax = std::max(lmax, l);
   };
   for (int64_t i = 0; i < n;) {
