@@ -531,7 +531,7 @@ static chns_status dirichlet_rows(const chns_mesh* m, int nc, const S* x, S* y, 
 
 chns_status apply_op(const chns_mesh* m, chns_operator op, const chns_params* prm,
                      const chns_coef* coef, const void* x, void* y, chns_precision prec,
-                     cudaStream_t s) {
+                     cudaStream_t s, bool zeroed) {
   CHNS_CHECK(m && prm && x && y, CHNS_EINVAL, "apply: null argument");
   CHNS_CHECK(op >= CHNS_OP_POISSON && op <= CHNS_OP_MOMENTUM, CHNS_EINVAL, "apply: bad operator");
   CHNS_CHECK(x != y, CHNS_EINVAL, "apply: x and y must not alias");
@@ -542,7 +542,7 @@ chns_status apply_op(const chns_mesh* m, chns_operator op, const chns_params* pr
   const int64_t n = nc * m->d.n_nodes;
   switch (prec) {
     case CHNS_FP64: {
-      CHNS_CUDA(cudaMemsetAsync(y, 0, n * sizeof(double), s));
+      if (!zeroed) CHNS_CUDA(cudaMemsetAsync(y, 0, n * sizeof(double), s));
       launch_apply<double, double, double>(m, op, p, coef_args<double>(coef),
                                            static_cast<const double*>(x), static_cast<double*>(y), s);
       if (op_dirichlet(op))
@@ -553,7 +553,7 @@ chns_status apply_op(const chns_mesh* m, chns_operator op, const chns_params* pr
       // double-float pays for the light operators (measured on 1.4e6 leaves: Poisson 0.76 ->
       // 0.31 ms, mass 1.01 -> 0.60 ms); the CH and momentum applies are faster in FP64 (1.90 vs
       // 1.96 ms, 7.8 vs 10.1 ms: register pressure and spills)
-      CHNS_CUDA(cudaMemsetAsync(y, 0, n * sizeof(double), s));
+      if (!zeroed) CHNS_CUDA(cudaMemsetAsync(y, 0, n * sizeof(double), s));
       if (op == CHNS_OP_POISSON || op == CHNS_OP_MASS)
         launch_apply_df(m, op, p, coef_args<double>(coef), static_cast<const double*>(x),
                         static_cast<double*>(y), s);
@@ -566,7 +566,7 @@ chns_status apply_op(const chns_mesh* m, chns_operator op, const chns_params* pr
       break;
     }
     case CHNS_FP32: {
-      CHNS_CUDA(cudaMemsetAsync(y, 0, n * sizeof(float), s));
+      if (!zeroed) CHNS_CUDA(cudaMemsetAsync(y, 0, n * sizeof(float), s));
       launch_apply<float, float, float>(m, op, p, coef_args<float>(coef),
                                         static_cast<const float*>(x), static_cast<float*>(y), s);
       if (op_dirichlet(op) && !tile_writes_rows(m, op))
@@ -574,7 +574,7 @@ chns_status apply_op(const chns_mesh* m, chns_operator op, const chns_params* pr
       break;
     }
     case CHNS_FP32_BF16COEF: {
-      CHNS_CUDA(cudaMemsetAsync(y, 0, n * sizeof(float), s));
+      if (!zeroed) CHNS_CUDA(cudaMemsetAsync(y, 0, n * sizeof(float), s));
       launch_apply<float, float, __nv_bfloat16>(m, op, p, coef_args<__nv_bfloat16>(coef),
                                                 static_cast<const float*>(x),
                                                 static_cast<float*>(y), s);
@@ -714,19 +714,20 @@ static DevParams shift_params(const chns_params* prm, double sa, double sb) {
 }
 
 chns_status apply_shift(const chns_mesh* m, const chns_params* prm, const void* phi, double sa,
-                        double sb, const void* x, void* y, chns_precision prec, cudaStream_t s) {
+                        double sb, const void* x, void* y, chns_precision prec, cudaStream_t s,
+                        bool zeroed) {
   CHNS_CHECK(m && prm && phi && x && y && x != y, CHNS_EINVAL, "shifted apply: bad argument");
   const DevParams p = shift_params(prm, sa, sb);
   chns_coef c{};
   c.phi_tilde = phi;
   const int64_t N = m->d.n_nodes;
   if (prec == CHNS_FP64) {
-    CHNS_CUDA(cudaMemsetAsync(y, 0, N * sizeof(double), s));
+    if (!zeroed) CHNS_CUDA(cudaMemsetAsync(y, 0, N * sizeof(double), s));
     launch_patch<ShiftK<double, double>, double, double, double, false>(
         m, p, coef_args<double>(&c), static_cast<const double*>(x), static_cast<double*>(y),
         nullptr, s);
   } else if (prec == CHNS_FP32) {
-    CHNS_CUDA(cudaMemsetAsync(y, 0, N * sizeof(float), s));
+    if (!zeroed) CHNS_CUDA(cudaMemsetAsync(y, 0, N * sizeof(float), s));
     if (use_tile<float, float>(m))
       launch_tile<TileShift, float, false>(m, p, coef_args<float>(&c),
                                            static_cast<const float*>(x), static_cast<float*>(y),

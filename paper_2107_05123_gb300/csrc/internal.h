@@ -174,9 +174,10 @@ constexpr int kMdMaxBlocks = 1024; // blocks of the GMRES multi-dot
 constexpr int kScalarBase = 3 * 4096;  // scalars stored after three partial arrays
 
 // ---- apply dispatch (apply.cu)
+// y = A x; zeroed: y is zero on entry (else it is cleared first: the applies add to it)
 chns_status apply_op(const chns_mesh* m, chns_operator op, const chns_params* prm,
                      const chns_coef* coef, const void* x, void* y, chns_precision prec,
-                     cudaStream_t s);
+                     cudaStream_t s, bool zeroed = false);
 // Slots of the CG scalars (offsets from the scalar area of ws.red). Iteration k (parity
 // par = k & 1) reads r.z of its iterate from kCgRz0 + par and that of the previous one from
 // kCgRzPrev, accumulates p.Ap into kCgPq0 + par, and accumulates the next r.z and r.r into
@@ -205,7 +206,8 @@ void momentum_qdata_off(const chns_mesh* m);
 // y = sa M x + sb K x (shifted Laplacian, constant sa, sb) and its exact diagonal; phi is any
 // coefficient array of the precision (FP64 or FP32), read but unused.
 chns_status apply_shift(const chns_mesh* m, const chns_params* prm, const void* phi, double sa,
-                        double sb, const void* x, void* y, chns_precision prec, cudaStream_t s);
+                        double sb, const void* x, void* y, chns_precision prec, cudaStream_t s,
+                        bool zeroed = false);
 chns_status diag_shift(const chns_mesh* m, const chns_params* prm, const void* phi, double sa,
                        double sb, void* d, chns_precision prec, cudaStream_t s);
 chns_status diag_op(const chns_mesh* m, chns_operator op, const chns_params* prm,

@@ -33,6 +33,17 @@ __device__ __forceinline__ void reduce_finalize(A (&v)[NV], double* __restrict__
   block_reduce_finalize<NV, kVecThreads>(v, part, kRedSlots, counter, out);
 }
 
+// Vector kernels that read several arrays and write others: kBatch elements per thread and round,
+// all of a round's loads before its first store (the compiler keeps the order of loads and stores
+// it cannot tell apart, which left one element's round trip to memory exposed per iteration).
+constexpr int kBatch = 4;
+#define BATCH_LOOP(i0, n)                                                    \
+  for (int64_t i0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i0 < (n); \
+       i0 += (int64_t)kBatch * gridDim.x * blockDim.x)
+#define BATCH(u, i, i0, n)                                                              \
+  _Pragma("unroll") for (int u = 0; u < kBatch; ++u)                                    \
+    if (const int64_t i = i0 + (int64_t)u * gridDim.x * blockDim.x; i < (n))
+
 #define GRID_LOOP(i, n)                                                     \
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < (n); \
        i += (int64_t)gridDim.x * blockDim.x)
@@ -166,15 +177,25 @@ k_cg_update(T* __restrict__ x, T* __restrict__ r, T* __restrict__ z, const T* __
             bool zero_q, int par) {
   const T a = cg_ratio<T>(S, kCgRz0 + par, kCgPq0 + par, true);
   typename Acc<T>::type v0 = Acc<T>::zero(), v1 = Acc<T>::zero();
-  GRID_LOOP(i, n) {
-    x[i] += a * p[i];
-    const T ri = r[i] - a * q[i];
-    if (zero_q) q[i] = T(0);
-    r[i] = ri;
-    const T zi = dinv ? dinv[i] * ri : ri;
-    z[i] = zi;
-    Acc<T>::fma(v0, ri, zi);
-    Acc<T>::fma(v1, ri, ri);
+  BATCH_LOOP(i0, n) {
+    T xv[kBatch], pv[kBatch], rv[kBatch], qv[kBatch], dv[kBatch];
+    BATCH(u, i, i0, n) {
+      xv[u] = x[i];
+      pv[u] = p[i];
+      rv[u] = r[i];
+      qv[u] = q[i];
+      dv[u] = dinv ? dinv[i] : T(1);
+    }
+    BATCH(u, i, i0, n) {
+      x[i] = xv[u] + a * pv[u];
+      const T ri = rv[u] - a * qv[u];
+      if (zero_q) q[i] = T(0);
+      r[i] = ri;
+      const T zi = dv[u] * ri;
+      z[i] = zi;
+      Acc<T>::fma(v0, ri, zi);
+      Acc<T>::fma(v1, ri, ri);
+    }
   }
   typename Acc<T>::type v[2] = {v0, v1};
   double tot[2];
@@ -223,11 +244,20 @@ k_fcg_update(T* __restrict__ x, T* __restrict__ r, const T* __restrict__ p,
              const T* __restrict__ q, int64_t n, double* __restrict__ S, int par) {
   const T a = cg_ratio<T>(S, kFcgRz0 + par, kCgPq0 + par, true);
   typename Acc<T>::type v0 = Acc<T>::zero();
-  GRID_LOOP(i, n) {
-    x[i] += a * p[i];
-    const T ri = r[i] - a * q[i];
-    r[i] = ri;
-    Acc<T>::fma(v0, ri, ri);
+  BATCH_LOOP(i0, n) {
+    T xv[kBatch], pv[kBatch], rv[kBatch], qv[kBatch];
+    BATCH(u, i, i0, n) {
+      xv[u] = x[i];
+      pv[u] = p[i];
+      rv[u] = r[i];
+      qv[u] = q[i];
+    }
+    BATCH(u, i, i0, n) {
+      x[i] = xv[u] + a * pv[u];
+      const T ri = rv[u] - a * qv[u];
+      r[i] = ri;
+      Acc<T>::fma(v0, ri, ri);
+    }
   }
   typename Acc<T>::type v[1] = {v0};
   double tot[1];
@@ -249,11 +279,18 @@ __global__ void __launch_bounds__(kVecThreads)
 k_fcg_dots(const T* __restrict__ z, T* __restrict__ q, const T* __restrict__ r, int64_t n,
            double* __restrict__ S, int par) {
   typename Acc<T>::type v0 = Acc<T>::zero(), v1 = Acc<T>::zero();
-  GRID_LOOP(i, n) {
-    const T zi = z[i];
-    Acc<T>::fma(v0, zi, q[i]);
-    q[i] = T(0);
-    Acc<T>::fma(v1, zi, r[i]);
+  BATCH_LOOP(i0, n) {
+    T zv[kBatch], qv[kBatch], rv[kBatch];
+    BATCH(u, i, i0, n) {
+      zv[u] = z[i];
+      qv[u] = q[i];
+      rv[u] = r[i];
+    }
+    BATCH(u, i, i0, n) {
+      q[i] = T(0);
+      Acc<T>::fma(v0, zv[u], qv[u]);
+      Acc<T>::fma(v1, zv[u], rv[u]);
+    }
   }
   typename Acc<T>::type v[2] = {v0, v1};
   double tot[2];
@@ -771,9 +808,9 @@ struct Snap {
 
 // Runs step(stream, it) — one iteration, which leaves r.r in S[kCgRr0 + ((it & 1) ^ 1)] — until
 // sqrt(r.r) <= tol_abs or max_it iterations; rr is r.r before the first iteration. With chunk >= 2 the iterations run
-// as CUDA graphs of `chunk` iterations (captured once per solve on a private stream); two graph
-// instances write r.r into alternating pinned host slots so the host checks chunk k while chunk
-// k+1 already runs. The solve may do up to two chunks beyond the iteration that reached the
+// as a CUDA graph of `chunk` iterations (captured once per solve on a private stream); after each
+// launch r.r is copied into one of two alternating pinned host slots, so the host checks chunk k
+// while chunk k+1 already runs. The solve may do up to two chunks beyond the iteration that reached the
 // tolerance; they only reduce the residual. Iteration parities are preserved (chunks are even).
 // With stall > 0 the iteration also stops (status CHNS_ENOTCONV) when the residual norm has not
 // halved over the last `stall` iterations (checked at the host checks).
@@ -825,49 +862,31 @@ chns_status iterate(const Ctx& c, Step&& step, T* x, double tol_abs, int max_it,
   } else if (std::sqrt(rr) > tol_abs && max_it > 0) {
     chunk += chunk & 1;  // even: every chunk starts at parity 0
     cudaStream_t cs = c.m->cap_stream;
-    cudaGraphExec_t ge[2] = {nullptr, nullptr};
+    cudaGraphExec_t ge = nullptr;
     cudaEvent_t ev[2] = {nullptr, nullptr};
     volatile double* slot = c.m->ws.h_pinned + 8;
     unsigned long long per_graph = 0;
     chns_status rc = CHNS_OK;
-    for (int v = 0; v < 2 && rc == CHNS_OK; ++v) {
-      cudaGraph_t g = nullptr;
-      cudaError_t e0 = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
-      if (e0 != cudaSuccess) {
-        rc = cuda_fail(e0, "cudaStreamBeginCapture");
-        break;
-      }
-      const unsigned long long l0 = chns_launches_now();
-      for (int i = 0; i < chunk && rc == CHNS_OK; ++i) rc = step(cs, i);
-      // an even chunk ends with an odd iteration, which leaves r.r in slot 0
-      cudaMemcpyAsync((void*)(slot + v), c.S + kCgRr0, sizeof(double), cudaMemcpyDeviceToHost, cs);
-      per_graph = chns_launches_now() - l0;
-      cudaError_t e1 = cudaStreamEndCapture(cs, &g);
-      if (rc != CHNS_OK) {
-        if (g) cudaGraphDestroy(g);
-        break;
-      }
-      // on a failure below, fall through to the cleanup loop so that the graph and event of
-      // the other instance are released too
-      if (e1 != cudaSuccess) {
-        rc = cuda_fail(e1, "cudaStreamEndCapture");
-        break;
-      }
-      cudaError_t e2 = cudaGraphInstantiate(&ge[v], g, 0);
-      cudaGraphDestroy(g);
-      if (e2 != cudaSuccess) {
-        ge[v] = nullptr;
-        rc = cuda_fail(e2, "cudaGraphInstantiate");
-        break;
-      }
-      cudaError_t e3 = cudaEventCreateWithFlags(&ev[v], cudaEventDisableTiming);
-      if (e3 != cudaSuccess) {
-        ev[v] = nullptr;
-        rc = cuda_fail(e3, "cudaEventCreateWithFlags");
-        break;
-      }
+    cudaGraph_t g = nullptr;
+    cudaError_t e0 = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
+    if (e0 != cudaSuccess) return cuda_fail(e0, "cudaStreamBeginCapture");
+    const unsigned long long l0 = chns_launches_now();
+    for (int i = 0; i < chunk && rc == CHNS_OK; ++i) rc = step(cs, i);
+    per_graph = chns_launches_now() - l0;
+    e0 = cudaStreamEndCapture(cs, &g);
+    if (rc == CHNS_OK && e0 != cudaSuccess) rc = cuda_fail(e0, "cudaStreamEndCapture");
+    if (rc == CHNS_OK && (e0 = cudaGraphInstantiate(&ge, g, 0)) != cudaSuccess) {
+      ge = nullptr;
+      rc = cuda_fail(e0, "cudaGraphInstantiate");
     }
-    note_launches_undo(2 * per_graph);  // captured, not executed
+    if (g) cudaGraphDestroy(g);
+    for (auto& v : ev)
+      if (rc == CHNS_OK &&
+          (e0 = cudaEventCreateWithFlags(&v, cudaEventDisableTiming)) != cudaSuccess) {
+        v = nullptr;
+        rc = cuda_fail(e0, "cudaEventCreateWithFlags");
+      }
+    note_launches_undo(per_graph);  // captured, not executed
     if (rc == CHNS_OK) {
       int k = 0;
       bool done = false;
@@ -878,8 +897,13 @@ chns_status iterate(const Ctx& c, Step&& step, T* x, double tol_abs, int max_it,
       };
       while (!done) {
         const int v = k & 1;
-        if (!ok(cudaGraphLaunch(ge[v], c.s), "cudaGraphLaunch")) break;
+        if (!ok(cudaGraphLaunch(ge, c.s), "cudaGraphLaunch")) break;
         note_launches(per_graph);
+        // an even chunk ends with an odd iteration, which leaves r.r in slot 0
+        if (!ok(cudaMemcpyAsync((void*)(slot + v), c.S + kCgRr0, sizeof(double),
+                                cudaMemcpyDeviceToHost, c.s),
+                "cudaMemcpyAsync"))
+          break;
         if (!ok(cudaEventRecord(ev[v], c.s), "cudaEventRecord")) break;
         it += chunk;
         // check the previous chunk while this one runs
@@ -896,10 +920,9 @@ chns_status iterate(const Ctx& c, Step&& step, T* x, double tol_abs, int max_it,
         ++k;
       }
     }
-    for (int v = 0; v < 2; ++v) {
-      if (ge[v]) cudaGraphExecDestroy(ge[v]);
-      if (ev[v]) cudaEventDestroy(ev[v]);
-    }
+    if (ge) cudaGraphExecDestroy(ge);
+    for (auto v : ev)
+      if (v) cudaEventDestroy(v);
     if (rc != CHNS_OK) return rc;
     if (!std::isfinite(rr)) {
       *iters = it;
@@ -992,8 +1015,22 @@ struct SchurPC {
   T* t[8] = {};          // scratch N-vectors: CG r, z, p, q, p2; t, w, u
   int itH = 20, itM = 5;
   chns_mg* mg = nullptr;  // when set, each H^-1 is one V-cycle of the shifted operator H
+  // From the kGraphAfter-th application on, the application (some 300 short launches) runs as a
+  // CUDA graph between two fixed vectors of the solve's workspace; the graph lives as long as
+  // this object, within one solve.
+  static constexpr int kGraphAfter = 2;
+  T *vin = nullptr, *vout = nullptr;  // 2N each
+  int applied = 0;
+  cudaGraphExec_t graph = nullptr;
+  unsigned long long graph_launches = 0;
+  SchurPC() = default;
+  SchurPC(const SchurPC&) = delete;
+  SchurPC& operator=(const SchurPC&) = delete;
+  ~SchurPC() {
+    if (graph) cudaGraphExecDestroy(graph);
+  }
 
-  // contexts and diagonals; vec: >= 10 scratch N-vectors
+  // contexts and diagonals; vec: 12 scratch N-vectors, 0 and 1, 10 and 11 contiguous
   chns_status setup(const Ctx& c, T* const* vec, int inner_its, chns_mg* hier = nullptr,
                     int mass_its = 0) {
     const int64_t N = c.m->d.n_nodes;
@@ -1013,6 +1050,8 @@ struct SchurPC {
     cK.sa = 0.0;
     cK.sb = kmu;
     for (int k = 0; k < 8; ++k) t[k] = vec[2 + k];
+    vin = vec[0];
+    vout = vec[10];
     const chns_precision pr = sizeof(T) == sizeof(double) ? CHNS_FP64 : CHNS_FP32;
     const void* phi = sizeof(T) == sizeof(double) ? c.coef64->phi_tilde : c.coefR.phi_tilde;
     mg = hier;
@@ -1048,6 +1087,36 @@ struct SchurPC {
 
   // z = P^-1 v for the pair [phi; mu] (2N each; z must not alias v)
   chns_status apply(const T* v, T* z) {
+    const size_t bytes = 2 * (size_t)cM.n * sizeof(T);
+    cudaStream_t s = cM.s;
+    if (applied++ < kGraphAfter) return launch(v, z);
+    if (!graph) {
+      cudaStream_t cs = cM.m->cap_stream;
+      CHNS_CUDA(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
+      const unsigned long long l0 = chns_launches_now();
+      cM.s = cH.s = cK.s = cs;
+      chns_status st = launch(vin, vout);
+      cM.s = cH.s = cK.s = s;
+      graph_launches = chns_launches_now() - l0;
+      note_launches_undo(graph_launches);  // captured, not executed
+      cudaGraph_t g = nullptr;
+      cudaError_t e = cudaStreamEndCapture(cs, &g);
+      if (st == CHNS_OK && e == cudaSuccess) e = cudaGraphInstantiate(&graph, g, 0);
+      if (g) cudaGraphDestroy(g);
+      if (st != CHNS_OK) return st;
+      if (e != cudaSuccess) {
+        graph = nullptr;
+        return cuda_fail(e, "Schur preconditioner graph");
+      }
+    }
+    CHNS_CUDA(cudaMemcpyAsync(vin, v, bytes, cudaMemcpyDeviceToDevice, s));
+    CHNS_CUDA(cudaGraphLaunch(graph, s));
+    note_launches(graph_launches);
+    CHNS_CUDA(cudaMemcpyAsync(z, vout, bytes, cudaMemcpyDeviceToDevice, s));
+    return CHNS_OK;
+  }
+
+  chns_status launch(const T* v, T* z) {
     const int64_t N = cM.n;
     const unsigned vg = vgrid(cM.m, N);
     const T* vphi = v;

@@ -59,11 +59,13 @@ __global__ void k_inject(const int32_t* __restrict__ inj, const T* __restrict__ 
 }
 
 // y[i] (+)= sum_k w[k] x[col[k]] over row i of a CSR table; with SUB the gathered values are
-// (x - x2)[col] (restriction of a residual r - A z formed on the fly)
+// (x - x2)[col] (restriction of a residual r - A z formed on the fly); clear (optional): set to
+// zero on the rows (the output of the next apply, which adds)
 template <class T, bool ADD, bool SUB>
 __global__ void k_csr_gather(const int32_t* __restrict__ ptr, const int32_t* __restrict__ col,
                              const float* __restrict__ w, const T* __restrict__ x,
-                             const T* __restrict__ x2, T* __restrict__ y, int64_t n) {
+                             const T* __restrict__ x2, T* __restrict__ y, int64_t n,
+                             T* __restrict__ clear = nullptr) {
   MG_LOOP(i, n) {
     T acc = T(0);
     const int b = ptr[i], e = ptr[i + 1];
@@ -73,32 +75,36 @@ __global__ void k_csr_gather(const int32_t* __restrict__ ptr, const int32_t* __r
       acc += (T)w[k] * v;
     }
     y[i] = ADD ? y[i] + acc : acc;
+    if (clear) clear[i] = T(0);
   }
 }
 
 // first Chebyshev step: d = f dinv (r - w) (w = A z of the current iterate, or absent for a
-// zero initial guess); z = d (zero guess) or z += d
+// zero initial guess); z = d (zero guess) or z += d; w is cleared for the next apply, which adds
+// (a memset launch per apply less)
 template <class T, bool GUESS>
 __global__ void k_cheb_first(const T* __restrict__ dinv, const T* __restrict__ r,
-                             const T* __restrict__ w, T* __restrict__ z, T* __restrict__ d, T f,
+                             T* __restrict__ w, T* __restrict__ z, T* __restrict__ d, T f,
                              int64_t n) {
   MG_LOOP(i, n) {
     const T ri = GUESS ? r[i] - w[i] : r[i];
     const T di = f * dinv[i] * ri;
     d[i] = di;
     z[i] = GUESS ? z[i] + di : di;
+    w[i] = T(0);
   }
 }
 
-// later Chebyshev steps: d = a d + b dinv (r - w); z += d
+// later Chebyshev steps: d = a d + b dinv (r - w); z += d; w cleared
 template <class T>
 __global__ void k_cheb_next(const T* __restrict__ dinv, const T* __restrict__ r,
-                            const T* __restrict__ w, T* __restrict__ z, T* __restrict__ d, T a, T b,
+                            T* __restrict__ w, T* __restrict__ z, T* __restrict__ d, T a, T b,
                             int64_t n) {
   MG_LOOP(i, n) {
     const T di = a * d[i] + b * dinv[i] * (r[i] - w[i]);
     d[i] = di;
     z[i] += di;
+    w[i] = T(0);
   }
 }
 
@@ -129,10 +135,13 @@ k_norm2(const T* __restrict__ v, int64_t n, double* __restrict__ slot) {
   if (threadIdx.x == 0) atomicAdd(slot, tot[0]);
 }
 
-// v /= sqrt(*slot)
+// v /= sqrt(*slot) (the FP64 root once per block, not per thread)
 template <class T>
 __global__ void k_normalise(T* __restrict__ v, const double* __restrict__ slot, int64_t n) {
-  const T s = (T)(1.0 / sqrt(slot[0]));
+  __shared__ T s_s;
+  if (threadIdx.x == 0) s_s = (T)(1.0 / sqrt(slot[0]));
+  __syncthreads();
+  const T s = s_s;
   MG_LOOP(i, n) v[i] *= s;
 }
 
@@ -204,32 +213,48 @@ __global__ void k_dense_assemble(MeshDev m, DevParams p, CoefArgs<double> cf,
 }
 
 // In-place Gauss-Jordan inverse of the SPD matrix A + c 1 1^T (no pivoting: the pivots of an SPD
-// matrix stay positive), one CTA.
-__global__ void __launch_bounds__(1024) k_gauss_jordan(double* __restrict__ A, int n, double c) {
-  __shared__ double colk[kMgMaxCoarse];
+// matrix stay positive), one CTA of 32 x 32 threads; in shared memory (in_smem) up to kGjSmem
+// rows. Bound by the FP64 pipe of its SM (n^2 operations per step at two per clock, 0.5 ms for
+// 125 rows; 1.2 ms when each step read and wrote the matrix in global memory and divided twice).
+constexpr int kGjSmem = 160;
+__global__ void __launch_bounds__(1024) k_gauss_jordan(double* __restrict__ A, int n, double c,
+                                                       bool in_smem) {
+  extern __shared__ __align__(16) double gj_smem[];
+  __shared__ double colk[kMgMaxCoarse], rowk[kMgMaxCoarse];
   __shared__ double piv_inv;
-  for (int64_t q = threadIdx.x; q < (int64_t)n * n; q += blockDim.x) A[q] += c;
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  double* M = in_smem ? gj_smem : A;
+  for (int i = ty; i < n; i += 32)
+    for (int j = tx; j < n; j += 32) M[i * n + j] = A[i * n + j] + c;
+  __syncthreads();
+  if (threadIdx.x == 0) piv_inv = 1.0 / M[0];
   __syncthreads();
   for (int k = 0; k < n; ++k) {
-    if (threadIdx.x == 0) piv_inv = 1.0 / A[(int64_t)k * n + k];
-    __syncthreads();
-    for (int j = threadIdx.x; j < n; j += blockDim.x) {
-      double* rk = A + (int64_t)k * n;
-      rk[j] = j == k ? piv_inv : rk[j] * piv_inv;
+    const double pi = piv_inv;
+    for (int j = threadIdx.x; j < n; j += 1024) {
+      rowk[j] = j == k ? pi : M[k * n + j] * pi;
+      colk[j] = M[j * n + k];
     }
-    for (int i = threadIdx.x; i < n; i += blockDim.x) colk[i] = A[(int64_t)i * n + k];
     __syncthreads();
-    const double* rk = A + (int64_t)k * n;
-    for (int64_t q = threadIdx.x; q < (int64_t)n * n; q += blockDim.x) {
-      const int i = (int)(q / n), j = (int)(q % n);
-      if (i == k) continue;
-      if (j == k)
-        A[q] = -colk[i] * piv_inv;
-      else
-        A[q] -= colk[i] * rk[j];
+    for (int i = ty; i < n; i += 32) {
+      const double ci = colk[i];
+      for (int j = tx; j < n; j += 32) {
+        const double rj = rowk[j];
+        double v;
+        if (i == k)
+          v = rj;
+        else if (j == k)
+          v = -ci * pi;
+        else
+          v = fma(-ci, rj, M[i * n + j]);
+        M[i * n + j] = v;
+        if (i == k + 1 && j == k + 1) piv_inv = 1.0 / v;  // of the next step
+      }
     }
     __syncthreads();
   }
+  if (in_smem)
+    for (int q = threadIdx.x; q < n * n; q += 1024) A[q] = M[q];
 }
 
 // z = C r for a dense n x n matrix, one warp per row
@@ -622,15 +647,17 @@ static const T* level_phi(chns_mg* g, int l) {
   return pick<T>(g->lv[l].op[kMgPoisson].phi64, g->lv[l].op[kMgPoisson].phi32);
 }
 
+// y = A x on level l; zeroed: y is zero already
 template <class T>
-static chns_status level_apply(chns_mg* g, int op, int l, const T* x, T* y, cudaStream_t s) {
+static chns_status level_apply(chns_mg* g, int op, int l, const T* x, T* y, cudaStream_t s,
+                               bool zeroed = false) {
   MgLevel& L = g->lv[l];
   if (op == kMgShifted)  // the patch kernel gathers one coefficient field, unused here
     return apply_shift(L.mesh, &g->phys, lv_dinv<T>(L, op), g->ops[op].sa, g->ops[op].sb, x, y,
-                       prec_of<T>(), s);
+                       prec_of<T>(), s, zeroed);
   chns_coef c{};
   c.phi_tilde = level_phi<T>(g, l);
-  return apply_op(L.mesh, CHNS_OP_POISSON, &g->phys, &c, x, y, prec_of<T>(), s);
+  return apply_op(L.mesh, CHNS_OP_POISSON, &g->phys, &c, x, y, prec_of<T>(), s, zeroed);
 }
 
 template <class T>
@@ -670,43 +697,70 @@ chns_status mg_setup_T(chns_mg* g, int op, cudaStream_t s) {
     chns_status st = level_diag<T>(g, op, l, s);
     if (st != CHNS_OK) return st;
   }
-  // largest eigenvalue of D^-1 A per level (power iteration, normalised on the device)
+  // The levels are independent of one another from here on: the coarsest inverse and the power
+  // iterations of the small levels (launch-bound) run on a second stream beside those of the two
+  // finest levels.
   const int NS = NL - 1;  // the coarsest level is solved exactly
-  double* slot = g->slots;
-  if (NS > 0) {
-    for (int l = 0; l < NS; ++l) {
-      MgLevel& L = g->lv[l];
-      note_launch();
-      k_power_start<T><<<grid_for(L.n), kMgThreads, 0, s>>>(lv_dinv<T>(L, op), lv_vec<T>(L, 3),
-                                                            L.n);
+  struct Fork {
+    cudaStream_t s, s2;
+    cudaEvent_t e = nullptr;
+    Fork(cudaStream_t a, cudaStream_t b) : s(a), s2(b) {}
+    chns_status order(cudaStream_t from, cudaStream_t to) {
+      if (!e) CHNS_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+      CHNS_CUDA(cudaEventRecord(e, from));
+      CHNS_CUDA(cudaStreamWaitEvent(to, e, 0));
+      return CHNS_OK;
     }
-    for (int it = 0; it <= g->prm.power_its; ++it) {
-      CHNS_CUDA(cudaMemsetAsync(slot, 0, NS * sizeof(double), s));
-      for (int l = 0; l < NS; ++l) {
-        MgLevel& L = g->lv[l];
-        T* v = lv_vec<T>(L, 3);
-        T* w = lv_vec<T>(L, 2);
+    ~Fork() {  // also after an error: nothing of the second stream outlives the call
+      order(s2, s);
+      if (e) cudaEventDestroy(e);
+    }
+  };
+  double* slot = g->slots;
+  {
+    Fork fork(s, g->lv.back().mesh->cap_stream);
+    CHNS_CUDA(cudaMemsetAsync(slot, 0, kMgMaxLevels * sizeof(double), s));
+    chns_status fst = fork.order(s, fork.s2);
+    if (fst != CHNS_OK) return fst;
+    // largest eigenvalue of D^-1 A on level l: power iteration, normalised every kNormEvery steps
+    // (the eigenvalues are of order one) and before the last, whose squared norm goes to the slot
+    constexpr int kNormEvery = 16;
+    auto power = [&](int l, cudaStream_t ps) -> chns_status {
+      MgLevel& L = g->lv[l];
+      T* v = lv_vec<T>(L, 3);
+      T* w = lv_vec<T>(L, 2);
+      note_launch();
+      k_power_start<T><<<grid_for(L.n), kMgThreads, 0, ps>>>(lv_dinv<T>(L, op), v, L.n);
+      const int K = g->prm.power_its;
+      for (int it = 0; it <= K; ++it) {
         if (it > 0) {
-          chns_status st = level_apply<T>(g, op, l, v, w, s);
+          chns_status st = level_apply<T>(g, op, l, v, w, ps);
           if (st != CHNS_OK) return st;
           note_launch();
-          k_mul<T><<<grid_for(L.n), kMgThreads, 0, s>>>(lv_dinv<T>(L, op), w, v, L.n);
+          k_mul<T><<<grid_for(L.n), kMgThreads, 0, ps>>>(lv_dinv<T>(L, op), w, v, L.n);
         }
+        const bool last = it == K, norm = it == K - 1 || it % kNormEvery == 0;
+        if (!last && !norm) continue;
+        CHNS_CUDA(cudaMemsetAsync(slot + l, 0, sizeof(double), ps));
         note_launch();
-        k_norm2<T><<<grid_for(L.n), kMgThreads, 0, s>>>(v, L.n, slot + l);
+        k_norm2<T><<<grid_for(L.n), kMgThreads, 0, ps>>>(v, L.n, slot + l);
+        if (last) continue;
         note_launch();
-        k_normalise<T><<<grid_for(L.n), kMgThreads, 0, s>>>(v, slot + l, L.n);
+        k_normalise<T><<<grid_for(L.n), kMgThreads, 0, ps>>>(v, slot + l, L.n);
       }
+      return CHNS_OK;
+    };
+    for (int l = 0; l < std::min(NS, 2); ++l) {
+      chns_status st = power(l, s);
+      if (st != CHNS_OK) return st;
     }
-    CHNS_CUDA(cudaMemcpyAsync(g->h_slots, slot, NS * sizeof(double), cudaMemcpyDeviceToHost, s));
-  }
-  // coarsest: dense inverse in FP64 (Poisson: of A + 1 1^T / n, the mean-zero solution)
-  {
+    cudaStream_t cs = fork.s2;
+    // coarsest: dense inverse in FP64 (Poisson: of A + 1 1^T / n, the mean-zero solution)
     MgLevel& C = g->lv.back();
     const int n = (int)C.n;
     // the FP32 setup works in its own FP64 matrix, so that the FP64 inverse stays valid
     double* Aw = sizeof(T) == sizeof(double) ? O.cinv64 : g->cwork64;
-    CHNS_CUDA(cudaMemsetAsync(Aw, 0, (size_t)n * n * sizeof(double), s));
+    CHNS_CUDA(cudaMemsetAsync(Aw, 0, (size_t)n * n * sizeof(double), cs));
     DevParams p = make_dev_params(g->phys);
     CoefArgs<double> cf{};
     cf.phi_shift = 0.0f;
@@ -719,27 +773,38 @@ chns_status mg_setup_T(chns_mg* g, int op, cudaStream_t s) {
         // FP64 copy of the FP32 coefficients in the coarsest level's FP64 apply-output vector
         double* tmp = C.v64[2];
         note_launch();
-        k_convert<T, double><<<grid_for(n), kMgThreads, 0, s>>>(level_phi<T>(g, NL - 1), tmp, n);
+        k_convert<T, double><<<grid_for(n), kMgThreads, 0, cs>>>(level_phi<T>(g, NL - 1), tmp, n);
         phic = tmp;
       }
       cf.phi = phic;
       note_launch();
-      k_dense_assemble<PoissonK<double, double>><<<nb, 128, 0, s>>>(C.mesh->d, p, cf, Aw, n);
+      k_dense_assemble<PoissonK<double, double>><<<nb, 128, 0, cs>>>(C.mesh->d, p, cf, Aw, n);
     } else {
       p.d.sa = O.sa;
       p.d.sb = O.sb;
       cf.phi = C.v64[2];  // gathered, unused
       note_launch();
-      k_dense_assemble<ShiftK<double, double>><<<nb, 128, 0, s>>>(C.mesh->d, p, cf, Aw, n);
+      k_dense_assemble<ShiftK<double, double>><<<nb, 128, 0, cs>>>(C.mesh->d, p, cf, Aw, n);
     }
+    const bool in_smem = n <= kGjSmem;
+    const size_t smem = in_smem ? (size_t)n * n * sizeof(double) : 0;
+    if (in_smem)
+      CHNS_CUDA(cudaFuncSetAttribute(k_gauss_jordan, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     kGjSmem * kGjSmem * (int)sizeof(double)));
     note_launch();
-    k_gauss_jordan<<<1, 1024, 0, s>>>(Aw, n, op == kMgPoisson ? 1.0 / n : 0.0);
+    k_gauss_jordan<<<1, 1024, smem, cs>>>(Aw, n, op == kMgPoisson ? 1.0 / n : 0.0, in_smem);
     if (sizeof(T) == sizeof(float)) {
       note_launch();
-      k_convert<double, float><<<grid_for((int64_t)n * n), kMgThreads, 0, s>>>(
+      k_convert<double, float><<<grid_for((int64_t)n * n), kMgThreads, 0, cs>>>(
           Aw, O.cinv32, (int64_t)n * n);
     }
+    for (int l = 2; l < NS; ++l) {
+      chns_status st = power(l, cs);
+      if (st != CHNS_OK) return st;
+    }
   }
+  if (NS > 0)
+    CHNS_CUDA(cudaMemcpyAsync(g->h_slots, slot, NS * sizeof(double), cudaMemcpyDeviceToHost, s));
   CHNS_CUDA(cudaGetLastError());
   CHNS_CUDA(cudaStreamSynchronize(s));
   for (int l = 0; l < NS; ++l) {
@@ -774,20 +839,21 @@ static chns_status vcycle(chns_mg* g, int op, int l, const T* r, T* z, cudaStrea
   T* w = lv_vec<T>(L, 2);
   T* d = lv_vec<T>(L, 3);
   chns_status st;
+  // every smoothing kernel leaves w zero, and so does the prolongation: no apply needs a memset
   auto smooth = [&](bool guess) -> chns_status {
     if (guess) {
-      st = level_apply<T>(g, op, l, z, w, s);
+      st = level_apply<T>(g, op, l, z, w, s, true);
       if (st != CHNS_OK) return st;
       note_launch();
       k_cheb_first<T, true><<<vg, kMgThreads, 0, s>>>(dinv, r, w, z, d, (T)(1.0 / theta), n);
     } else {
       note_launch();
-      k_cheb_first<T, false><<<vg, kMgThreads, 0, s>>>(dinv, r, nullptr, z, d, (T)(1.0 / theta), n);
+      k_cheb_first<T, false><<<vg, kMgThreads, 0, s>>>(dinv, r, w, z, d, (T)(1.0 / theta), n);
     }
     double rho_old = 1.0 / sigma;
     for (int i = 1; i < g->prm.degree; ++i) {
       const double rho = 1.0 / (2.0 * sigma - rho_old);
-      st = level_apply<T>(g, op, l, z, w, s);
+      st = level_apply<T>(g, op, l, z, w, s, true);
       if (st != CHNS_OK) return st;
       note_launch();
       k_cheb_next<T><<<vg, kMgThreads, 0, s>>>(dinv, r, w, z, d, (T)(rho * rho_old),
@@ -798,7 +864,7 @@ static chns_status vcycle(chns_mg* g, int op, int l, const T* r, T* z, cudaStrea
   };
   if ((st = smooth(false)) != CHNS_OK) return st;
   // coarse correction: r_c = R (r - A z), z += P z_c
-  if ((st = level_apply<T>(g, op, l, z, w, s)) != CHNS_OK) return st;
+  if ((st = level_apply<T>(g, op, l, z, w, s, true)) != CHNS_OK) return st;
   MgLevel& Cl = g->lv[l + 1];
   T* rc = lv_vec<T>(Cl, 0);
   T* zc = lv_vec<T>(Cl, 1);
@@ -808,7 +874,7 @@ static chns_status vcycle(chns_mg* g, int op, int l, const T* r, T* z, cudaStrea
   if ((st = vcycle<T>(g, op, l + 1, rc, zc, s)) != CHNS_OK) return st;
   note_launch();
   k_csr_gather<T, true, false><<<vg, kMgThreads, 0, s>>>(L.p_ptr, L.p_col, L.p_w, zc, nullptr, z,
-                                                         n);
+                                                         n, w);
   if ((st = smooth(true)) != CHNS_OK) return st;
   CHNS_CUDA(cudaGetLastError());
   return CHNS_OK;
