@@ -1293,10 +1293,8 @@ chns_status gmres(const Ctx& c, const T* b, T* x, const T* dinv, bool block2, do
         if (x) cudaEventDestroy(x);
     }
   } ev;
-  if (fused) {
+  if (fused)
     for (auto& x : ev.e) CHNS_CUDA(cudaEventCreateWithFlags(&x, cudaEventDisableTiming));
-    CHNS_CUDA(cudaMemsetAsync(arnoldi_acc(c, 0), 0, kArnoldiBytes, c.s));
-  }
   auto Hij = [&](int i, int j) -> double& { return H[(size_t)i * restart + j]; };
   for (;;) {
     // r = b - A x into V_0
@@ -1316,6 +1314,9 @@ chns_status gmres(const Ctx& c, const T* b, T* x, const T* dinv, bool block2, do
     if (beta <= tol_abs || it >= max_it) break;
     note_launch();
     k_scale<T><<<vg, kVecThreads, 0, c.s>>>(V, 1.0 / beta, n);
+    // a cycle starts at parity 0, whose sums and barrier the last column of the cycle before may
+    // have used
+    if (fused) CHNS_CUDA(cudaMemsetAsync(arnoldi_acc(c, 0), 0, kArnoldiBytes, c.s));
     std::fill(g.begin(), g.end(), 0.0);
     g[0] = beta;
     int jend = 0;
