@@ -252,8 +252,13 @@ static void launch_tile(const chns_mesh* m, const DevParams& p, const CoefArgs<C
                         const float* x, float* y, double* S_cg, cudaStream_t s,
                         const float* z = nullptr, float* pout = nullptr, int par = 0, int fcg = 0) {
   constexpr size_t smem =
-      (size_t)((kTileThreads / 32 + 1) * Op::NC + (Op::FIELD ? 1 : 0)) * kPatchSlots * 4;
+      (size_t)((kTileThreads / 32 + 1) * Op::NC + Op::NF) * kPatchSlots * 4;
   auto* fn = k_apply_tile<Op, C, CGP>;
+  if constexpr (smem > 48 * 1024) {
+    static const cudaError_t configured =
+        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    (void)configured;
+  }
   int64_t grid = std::min(m->d.n_patch, (int64_t)Op::CTAS * std::max(m->sm_count, 1));
   if (m->apply_max_ctas > 0) grid = std::min(grid, m->apply_max_ctas);
   note_launch();
@@ -267,17 +272,19 @@ static void launch_tile(const chns_mesh* m, const DevParams& p, const CoefArgs<C
 // a CUDA graph, Poisson, per-patch / this: 2,878 leaves 5.9 / 6.6 us, 77,932 7.1 / 7.5, 156,640
 // 8.4 / 8.5, 314,672 (8.2 patches per SM) 13.4 / 12.5, 1,429,744 40.4 / 34.6).
 constexpr int kTilePatchesPerSm = 8;
+// The momentum apply is faster in it on every mesh (see TileMom).
 template <class T, class S>
-static bool use_tile(const chns_mesh* m) {
+static bool use_tile(const chns_mesh* m, chns_operator op) {
   if (!(std::is_same<T, float>::value && std::is_same<S, float>::value)) return false;
   if (m->apply_kernel == CHNS_APPLY_PATCH) return false;
   if (m->apply_kernel == CHNS_APPLY_STREAM) return true;
-  return m->d.n_patch >= (int64_t)kTilePatchesPerSm * std::max(m->sm_count, 1);
+  const int from = op == CHNS_OP_MOMENTUM ? 0 : kTilePatchesPerSm;
+  return m->d.n_patch >= (int64_t)from * std::max(m->sm_count, 1);
 }
 
 // Operators whose FP32 two-leaves-per-thread kernel also writes the identity rows.
 static bool tile_writes_rows(const chns_mesh* m, chns_operator op) {
-  return op == CHNS_OP_MASS && use_tile<float, float>(m);
+  return (op == CHNS_OP_MASS || op == CHNS_OP_MOMENTUM) && use_tile<float, float>(m, op);
 }
 
 // Reference (corner a, slot k) -> node reference with Dirichlet bit and its weight, or -1.
@@ -413,7 +420,7 @@ static void launch_apply(const chns_mesh* m, chns_operator op, const DevParams& 
   switch (op) {
     case CHNS_OP_POISSON:
       if constexpr (std::is_same<T, float>::value && std::is_same<S, T>::value) {
-        if (use_tile<T, S>(m)) {
+        if (use_tile<T, S>(m, op)) {
           launch_tile<TilePoisson<false>, C, false>(m, p, cf, x, y, nullptr, s);
           break;
         }
@@ -422,7 +429,7 @@ static void launch_apply(const chns_mesh* m, chns_operator op, const DevParams& 
       break;
     case CHNS_OP_MASS:
       if constexpr (std::is_same<T, float>::value && std::is_same<S, T>::value) {
-        if (use_tile<T, S>(m)) {
+        if (use_tile<T, S>(m, op)) {
           launch_tile<TileMass, C, false>(m, p, cf, x, y, nullptr, s);
           break;
         }
@@ -438,10 +445,22 @@ static void launch_apply(const chns_mesh* m, chns_operator op, const DevParams& 
       if (m->mq.on && qd) {
         CoefArgs<C> cq = cf;
         cq.qd = qd;
+        if constexpr (std::is_same<T, float>::value && std::is_same<S, T>::value) {
+          if (use_tile<T, S>(m, op)) {
+            launch_tile<TileMomQ, C, false>(m, p, cq, x, y, nullptr, s);
+            break;
+          }
+        }
         launch_patch<MomQK<T, C>, T, S, C, false>(m, p, cq, x, y, nullptr, s);
-      } else {
-        launch_patch<MomK<T, C>, T, S, C, false>(m, p, cf, x, y, nullptr, s);
+        break;
       }
+      if constexpr (std::is_same<T, float>::value && std::is_same<S, T>::value) {
+        if (use_tile<T, S>(m, op)) {
+          launch_tile<TileMom, C, false>(m, p, cf, x, y, nullptr, s);
+          break;
+        }
+      }
+      launch_patch<MomK<T, C>, T, S, C, false>(m, p, cf, x, y, nullptr, s);
       break;
     }
   }
@@ -671,7 +690,7 @@ chns_status apply_poisson_cg(const chns_mesh* m, const chns_params* prm, const c
           static_cast<double*>(p_new), par, fcg);
       break;
     case CHNS_FP32:
-      if (use_tile<float, float>(m)) {
+      if (use_tile<float, float>(m, CHNS_OP_POISSON)) {
         launch_tile<TilePoisson<true>, float, true>(
             m, p, coef_args<float>(coef), static_cast<const float*>(p_old), static_cast<float*>(y),
             S_cg, s, static_cast<const float*>(z), static_cast<float*>(p_new), par, fcg);
@@ -682,7 +701,7 @@ chns_status apply_poisson_cg(const chns_mesh* m, const chns_params* prm, const c
           S_cg, s, static_cast<const float*>(z), static_cast<float*>(p_new), par, fcg);
       break;
     case CHNS_FP32_BF16COEF:
-      if (use_tile<float, float>(m)) {
+      if (use_tile<float, float>(m, CHNS_OP_POISSON)) {
         launch_tile<TilePoisson<true>, __nv_bfloat16, true>(
             m, p, coef_args<__nv_bfloat16>(coef), static_cast<const float*>(p_old),
             static_cast<float*>(y), S_cg, s, static_cast<const float*>(z),
@@ -728,7 +747,7 @@ chns_status apply_shift(const chns_mesh* m, const chns_params* prm, const void* 
         nullptr, s);
   } else if (prec == CHNS_FP32) {
     if (!zeroed) CHNS_CUDA(cudaMemsetAsync(y, 0, N * sizeof(float), s));
-    if (use_tile<float, float>(m))
+    if (use_tile<float, float>(m, CHNS_OP_POISSON))
       launch_tile<TileShift, float, false>(m, p, coef_args<float>(&c),
                                            static_cast<const float*>(x), static_cast<float*>(y),
                                            nullptr, s);

@@ -445,6 +445,91 @@ struct Kron {
   }
 };
 
+// ---- the same in packed FP32 for one element: pairs over the Gauss points (or corners) along x,
+// so that half the instructions do the work without a second element's registers. Index j = y + 2 z
+// of the four x lines; the x stage is scalar, its two results land in one pair.
+template <bool NORM>
+__device__ __forceinline__ F2 it_x(float a, float b) {
+  F2 o;
+  interp<NORM>(a, b, o.x, o.y);
+  return o;
+}
+template <bool NORM>
+__device__ __forceinline__ void interp_yz(const F2 t[4], F2 v[4]) {
+  F2 s[4];
+#pragma unroll
+  for (int z = 0; z < 4; z += 2) interp<NORM>(t[z], t[z + 1], s[z], s[z + 1]);
+#pragma unroll
+  for (int y = 0; y < 2; ++y) interp<NORM>(s[y], s[y + 2], v[y], v[y + 2]);
+}
+// corner values to the Gauss points
+template <bool NORM>
+__device__ __forceinline__ void interp3(const float u[8], F2 v[4]) {
+  F2 t[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) t[j] = it_x<NORM>(u[2 * j], u[2 * j + 1]);
+  interp_yz<NORM>(t, v);
+}
+// the transpose
+template <bool NORM>
+__device__ __forceinline__ void interp3_t(const F2 v[4], F2 r[4]) {
+  F2 t[4];
+  interp_yz<NORM>(v, t);
+#pragma unroll
+  for (int j = 0; j < 4; ++j) r[j] = it_x<NORM>(t[j].x, t[j].y);
+}
+
+// GradC in pairs along x
+struct GradP {
+  float x[4];     // [qy + 2 qz]
+  F2 y[2], z[2];  // [qz], [qy]
+  __device__ __forceinline__ void eval(const float u[8], const float c[3]) {
+    float d[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) d[j] = u[2 * j + 1] - u[2 * j];
+    interp2(d, x);
+    F2 l[4], t0, t1;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) l[j] = F2(u[2 * j], u[2 * j + 1]);
+    it(l[1] - l[0], l[3] - l[2], t0, t1);
+    y[0] = F2(c[1]) * it_x<false>(t0.x, t0.y);
+    y[1] = F2(c[1]) * it_x<false>(t1.x, t1.y);
+    it(l[2] - l[0], l[3] - l[1], t0, t1);
+    z[0] = F2(c[2]) * it_x<false>(t0.x, t0.y);
+    z[1] = F2(c[2]) * it_x<false>(t1.x, t1.y);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) x[j] *= c[0];
+  }
+  __device__ __forceinline__ F2 at(int j, int d) const {
+    return d == 0 ? F2(x[j]) : d == 1 ? y[j >> 1] : z[j & 1];
+  }
+  __device__ __forceinline__ void sum(int j, int d, F2 v) {
+    if (d == 0)
+      x[j] = v.x + v.y;
+    else if (d == 1)
+      y[j >> 1] = j & 1 ? y[j >> 1] + v : v;
+    else
+      z[j & 1] = j & 2 ? z[j & 1] + v : v;
+  }
+  __device__ __forceinline__ void transpose(const float sc[3], F2 r[4]) const {
+    float t[4];
+    interp2(x, t);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) r[j] = F2(fmaf(-sc[0], t[j], r[j].x), fmaf(sc[0], t[j], r[j].y));
+    F2 a, b;
+    it(it_x<false>(y[0].x, y[0].y), it_x<false>(y[1].x, y[1].y), a, b);  // z = 0, 1
+    r[1] = mad(F2(sc[1]), a, r[1]);
+    r[0] = mad(F2(-sc[1]), a, r[0]);
+    r[3] = mad(F2(sc[1]), b, r[3]);
+    r[2] = mad(F2(-sc[1]), b, r[2]);
+    it(it_x<false>(z[0].x, z[0].y), it_x<false>(z[1].x, z[1].y), a, b);  // y = 0, 1
+    r[2] = mad(F2(sc[2]), a, r[2]);
+    r[0] = mad(F2(-sc[2]), a, r[0]);
+    r[3] = mad(F2(sc[2]), b, r[3]);
+    r[1] = mad(F2(-sc[2]), b, r[1]);
+  }
+};
+
 // Compile-time loop over the 8 quadrature points.
 template <int Q = 0, class F>
 __device__ __forceinline__ void for_qp(F&& f) {

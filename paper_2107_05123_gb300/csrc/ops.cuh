@@ -399,6 +399,105 @@ __device__ __forceinline__ void momentum_apply(const Geo<T>& g, const T x[3][8],
   }
 }
 
+// The same in packed FP32: the pair of Gauss points along x of line j = qy + 2 qz at once.
+__device__ __forceinline__ VmsQ<F2> vms_point(F2 pv, const F2 gp[3], const F2 j[3], const F2 u[3],
+                                              const VmsElem<float>& el, const PrmT<float>& k) {
+  VmsQ<F2> o;
+  const F2 pc = clamp_nan(pv, -1.f, 1.f);
+  o.rho = mad(F2(k.alpha), pc, F2(k.beta));
+  const F2 eta = mad(F2(k.gamma), pc, F2(k.xi));
+  const float gge = k.h2re * k.gamma;
+  o.gge = F2(inside1(pv.x) ? gge : 0.f, inside1(pv.y) ? gge : 0.f);
+  o.ir = F2(recip(o.rho.x), recip(o.rho.y));
+  F2 ugu(k.four_idt2), ugj(0.f);
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    const F2 gu = F2(el.G[d]) * u[d];
+    ugu = mad(gu, u[d], ugu);
+    ugj = d == 0 ? gu * j[d] : mad(gu, j[d], ugj);
+  }
+  const F2 er = eta * o.ir;
+  const F2 rad = mad(F2(2.f) * o.ir, ugj, mad(er * er, F2(el.visc), ugu));
+  o.tau = F2(inv_sqrt(rad.x > k.four_idt2 ? rad.x : k.four_idt2),
+             inv_sqrt(rad.y > k.four_idt2 ? rad.y : k.four_idt2));
+  o.a0 = o.rho * F2(k.idt);
+  o.e = eta * F2(k.h2re);
+  const F2 hr = F2(0.5f) * o.rho, ht = F2(0.5f) * o.tau, ti = o.tau * o.ir;
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    o.b[d] = mad(hr, u[d], j[d]);
+    o.bp[d] = mad(-o.gge, gp[d], o.b[d]);
+    o.t[d] = mad(ht, u[d], ti * j[d]);
+  }
+  return o;
+}
+
+struct VmsFieldsP {
+  F2 pv[4], uq[3][4];
+  GradP gp, gj;
+  __device__ __forceinline__ void eval(const float pe[8], const float me[8], const float ue[3][8],
+                                       const Geo<float>& g, const PrmT<float>& k) {
+    constexpr double w = gauss_w<float>();
+    const float w2 = (float)(w * w), wj = w2 * k.h2pe * k.ka;
+    const float cp[3] = {w2 * g.ih[0], w2 * g.ih[1], w2 * g.ih[2]};
+    const float cj[3] = {wj * g.ih[0], wj * g.ih[1], wj * g.ih[2]};
+    interp3<true>(pe, pv);
+    gp.eval(pe, cp);
+    gj.eval(me, cj);
+#pragma unroll
+    for (int d = 0; d < 3; ++d) interp3<true>(ue[d], uq[d]);
+  }
+  __device__ __forceinline__ VmsQ<F2> at(int q, const VmsElem<float>& el,
+                                         const PrmT<float>& k) const {
+    const F2 p[3] = {gp.at(q, 0), gp.at(q, 1), gp.at(q, 2)};
+    const F2 j[3] = {gj.at(q, 0), gj.at(q, 1), gj.at(q, 2)};
+    const F2 u[3] = {uq[0][q], uq[1][q], uq[2][q]};
+    return vms_point(pv[q], p, j, u, el, k);
+  }
+};
+
+// coef(j, ...) gives the coefficients of the point pair j
+template <class F>
+__device__ __forceinline__ void momentum_apply_pairs(const Geo<float>& g, const float x[3][8],
+                                                     float r[3][8], F&& coef) {
+  constexpr double w = gauss_w<float>();
+  const float cg[3] = {(float)(w * w) * g.ih[0], (float)(w * w) * g.ih[1],
+                       (float)(w * w) * g.ih[2]};
+  F2 v[3][4];
+  GradP d[3], s[3];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    interp3<true>(x[k], v[k]);
+    d[k].eval(x[k], cg);
+  }
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    F2 a0, b[3], bp[3], e, t[3];
+    coef(q, a0, b, bp, e, t);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const F2 vg[3] = {d[k].at(q, 0), d[k].at(q, 1), d[k].at(q, 2)};
+      const F2 av = a0 * v[k][q];
+      const F2 R = mad(bp[0], vg[0], mad(bp[1], vg[1], mad(bp[2], vg[2], av)));
+      v[k][q] = F2(g.detJ) * mad(b[0], vg[0], mad(b[1], vg[1], mad(b[2], vg[2], av)));
+#pragma unroll
+      for (int i = 0; i < 3; ++i) s[k].sum(q, i, mad(R, t[i], e * vg[i]));
+    }
+  }
+  const float sc[3] = {g.detJ * cg[0], g.detJ * cg[1], g.detJ * cg[2]};
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    F2 o[4];
+    interp3_t<true>(v[k], o);
+    s[k].transpose(sc, o);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      r[k][2 * j] = o[j].x;
+      r[k][2 * j + 1] = o[j].y;
+    }
+  }
+}
+
 template <class T, class C>
 struct MomK {
   static constexpr bool QDATA = false;

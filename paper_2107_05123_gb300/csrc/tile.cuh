@@ -5,8 +5,9 @@
 // of the adaptive workloads) or any two other leaves.
 //  1. the values of the regular slots go to shared memory, then the hanging slots are
 //     interpolated (mean of 2 or 4 parents);
-//  2. each thread applies the element operator to its two leaves at once, sum-factorised, in
-//     packed FP32 pairs (one issue slot for two operations);
+//  2. each thread applies the element operator to its two leaves, sum-factorised, in packed FP32 pairs
+//     (one issue slot for two operations): Poisson, mass and shifted to both leaves at once,
+//     momentum to one after the other with pairs of Gauss points;
 //  3. the contributions are added to sums per slot in shared memory, one array per warp, by plain
 //     read-add-write: the threads of a warp add the same corner of their leaves in the same step,
 //     and a point is that corner of at most one leaf (the one that fills that octant around it),
@@ -250,13 +251,20 @@ struct PairConst {
 };
 
 // ---------------------------------------------------------------- operators
-// NC components; FIELD: one coefficient field s = 1 + phi~; consts(): four constants of a level.
-// setup() computes what the components share, apply() the contributions of one component.
+// NC components; NF coefficient fields: phi~ (ONE_PLUS: s = 1 + phi~), then the velocity, then mu~;
+// consts(): four constants of a level; AHEAD: the next patch's values are loaded while a patch is
+// computed. setup() computes what the components share and apply() the contributions of one
+// component of a thread's two leaves at once (kPair); or leaf() computes one leaf after the other
+// (kLeaf), in packed pairs of Gauss points, for operators whose state would not fit the registers
+// twice.
+enum class TileForm { kPair, kLeaf };
 // "Columns" are the x lines here: the first stage runs along x, the in-plane axes are y and z.
 template <bool E>
 struct TilePoisson {
   static constexpr int NC = 1;
-  static constexpr bool FIELD = true, DIR = false, ENERGY = E;
+  static constexpr int NF = 1;
+  static constexpr bool ONE_PLUS = true, AHEAD = true, DIR = false, ENERGY = E;
+  static constexpr TileForm FORM = TileForm::kPair;
   static constexpr int CTAS = 7;  // resident CTAs per SM the register allocation allows
   static __device__ __forceinline__ float4 consts(const LevelGeo& g, const PrmT<float>&) {
     const float d = g.detJf * (float)(kWr2 * kWr2);
@@ -290,7 +298,9 @@ struct TilePoisson {
 // (w, rho~ u) per component
 struct TileMass {
   static constexpr int NC = 3;
-  static constexpr bool FIELD = true, DIR = true, ENERGY = false;
+  static constexpr int NF = 1;
+  static constexpr bool ONE_PLUS = true, AHEAD = true, DIR = true, ENERGY = false;
+  static constexpr TileForm FORM = TileForm::kPair;
   static constexpr int CTAS = 5;
   static __device__ __forceinline__ float4 consts(const LevelGeo& g, const PrmT<float>&) {
     return make_float4(g.detJf, 0.f, 0.f, 0.f);
@@ -324,7 +334,9 @@ struct TileMass {
 // E = Py Dx u.
 struct TileShift {
   static constexpr int NC = 1;
-  static constexpr bool FIELD = false, DIR = false, ENERGY = false;
+  static constexpr int NF = 0;
+  static constexpr bool ONE_PLUS = false, AHEAD = true, DIR = false, ENERGY = false;
+  static constexpr TileForm FORM = TileForm::kPair;
   static constexpr int CTAS = 7;
   static __device__ __forceinline__ float4 consts(const LevelGeo& g, const PrmT<float>& k) {
     const float V = 8.f * g.detJf, ks = k.sb * V * (float)(1.0 / 36.0);
@@ -381,6 +393,108 @@ struct TileShift {
   }
 };
 
+// constants of a level for the operators in leaf form, and what they are
+__device__ __forceinline__ float4 leaf_consts(const LevelGeo& g) {
+  return make_float4(g.detJf, g.ihf[0], g.ihf[1], g.ihf[2]);
+}
+__device__ __forceinline__ Geo<float> leaf_geometry(const float4& c) {
+  Geo<float> g;
+  g.detJ = c.x;
+  g.ih[0] = c.y;
+  g.ih[1] = c.z;
+  g.ih[2] = c.w;
+  return g;
+}
+
+// The momentum operator with its coefficients evaluated on the fly (see MomK), one leaf after the
+// other in packed pairs of Gauss points. Bound by latency (as CTA-per-patch kernel: 34 % of the issue
+// slots, barriers 25 % and loads of the gather 20 % of the stalls): three CTAs of four warps at 168
+// registers overlap their phases better than two of eight at 128, and the sums need no
+// compare-and-swap loops, 24 per leaf. FP32 in a CUDA graph, CTA-per-patch kernel / this: 1,429,744
+// leaves 217 / 143 us, 314,672 48.0 / 36.5, 77,932 19.6 / 15.6, 19,608 12.6 / 11.8; four CTAs at 128
+// registers 194 us on the first (412 bytes of spills), in scalar arithmetic 178 us.
+struct TileMom {
+  static constexpr int NC = 3;
+  static constexpr int NF = 5;  // phi~, u_hat, mu~
+  static constexpr bool ONE_PLUS = false, AHEAD = false, DIR = true, ENERGY = false;
+  static constexpr TileForm FORM = TileForm::kLeaf;
+  static constexpr int CTAS = 3;
+  static __device__ __forceinline__ float4 consts(const LevelGeo& g, const PrmT<float>&) {
+    return leaf_consts(g);
+  }
+  template <class At>
+  static __device__ __forceinline__ void leaf(const float4& c, const PrmT<float>& k, const float* xs,
+                                              const float* fs, const At& at, const float*, int64_t,
+                                              float (&r)[NC][8]) {
+    const Geo<float> g = leaf_geometry(c);
+    VmsFieldsP f;
+    {
+      float pe[8], me[8], ue[3][8];
+#pragma unroll
+      for (int a = 0; a < 8; ++a) {
+        pe[a] = at(fs, a);
+#pragma unroll
+        for (int d = 0; d < 3; ++d) ue[d][a] = at(fs + (1 + d) * kPatchSlots, a);
+        me[a] = at(fs + 4 * kPatchSlots, a);
+      }
+      f.eval(pe, me, ue, g, k);
+    }
+    float x[NC][8];
+#pragma unroll
+    for (int n = 0; n < NC; ++n)
+#pragma unroll
+      for (int a = 0; a < 8; ++a) x[n][a] = at(xs + n * kPatchSlots, a);
+    const VmsElem<float> el(g, k);
+    momentum_apply_pairs(g, x, r, [&](int q, F2& a0, F2 b[3], F2 bp[3], F2& e, F2 t[3]) {
+      const VmsQ<F2> v = f.at(q, el, k);
+      a0 = v.a0;
+      e = v.e;
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        b[d] = v.b[d];
+        bp[d] = v.bp[d];
+        t[d] = v.t[d];
+      }
+    });
+  }
+};
+
+// The momentum operator from quadrature data (see MomQK), likewise.
+struct TileMomQ {
+  static constexpr int NC = 3;
+  static constexpr int NF = 0;
+  static constexpr bool ONE_PLUS = false, AHEAD = false, DIR = true, ENERGY = false;
+  static constexpr TileForm FORM = TileForm::kLeaf;
+  static constexpr int CTAS = 3;
+  static __device__ __forceinline__ float4 consts(const LevelGeo& g, const PrmT<float>&) {
+    return leaf_consts(g);
+  }
+  // qd: of this leaf
+  template <class At>
+  static __device__ __forceinline__ void leaf(const float4& c, const PrmT<float>&, const float* xs,
+                                              const float*, const At& at, const float* qd, int64_t ne,
+                                              float (&r)[NC][8]) {
+    const Geo<float> g = leaf_geometry(c);
+    float x[NC][8];
+#pragma unroll
+    for (int n = 0; n < NC; ++n)
+#pragma unroll
+      for (int a = 0; a < 8; ++a) x[n][a] = at(xs + n * kPatchSlots, a);
+    momentum_apply_pairs(g, x, r, [&](int q, F2& a0, F2 b[3], F2 bp[3], F2& e, F2 t[3]) {
+      const float* p = qd + (int64_t)(2 * q) * kMomQ * ne;
+      auto pair = [&](int v) { return F2(__ldg(p + v * ne), __ldg(p + (v + kMomQ) * ne)); };
+      a0 = pair(0);
+      e = pair(7);
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        b[d] = pair(1 + d);
+        bp[d] = pair(4 + d);
+        t[d] = pair(8 + d);
+      }
+    });
+  }
+};
+
 // ---------------------------------------------------------------- kernel
 constexpr int kPreSlots = 3;  // regular slots per thread whose values are loaded ahead
 constexpr int kPreHang = 2;   // hanging slots per thread whose parents are loaded ahead
@@ -390,28 +504,80 @@ constexpr int kPreHang = 2;   // hanging slots per thread whose parents are load
 template <int NA>
 struct TilePre {
   uint32_t id[kPreSlots];
-  float v[kPreSlots][NA];  // components (CGP: p_old and z of the component), then s
+  float v[kPreSlots][NA];  // components (CGP: p_old and z of the component), then fields
   uint2 par[kPreHang];
   uint32_t ref[8];
 };
+
+// A thread's two leaves one after the other (kLeaf). Bricks and other leaves need no separate steps:
+// every thread adds corner a of its leaf in step a.
+template <class Op>
+__device__ __forceinline__ void tile_leaves(const PrmT<float>& k, const uint32_t ref[8],
+                                            const float4* cst, bool brick, bool any,
+                                            const float* xs, const float* fs, const float* qd,
+                                            int64_t ne, float* yw) {
+  const PairRefs<true> pr{ref};
+  // byte offsets of the corners of both leaves, x = 0 | x = 1 << 16, per x line
+  uint32_t o0[4], o1[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const uint32_t a = brick ? pr(3 * j) : pr(2 * j), b = brick ? pr(3 * j + 1) : pr(2 * j + 1),
+                   c = brick ? b : pr(8 + 2 * j), d = brick ? pr(3 * j + 2) : pr(9 + 2 * j);
+    o0[j] = a | b << 16;
+    o1[j] = c | d << 16;
+  }
+  const bool two = any && (brick || pr.nibble(3) != 0);
+  const uint32_t l0 = pr.nibble(0), l1 = brick ? l0 : pr.nibble(4);
+  const uint32_t n0 = pr.nibble(1) | pr.nibble(2) << 4,
+                 n1 = brick ? n0 + 1 : pr.nibble(5) | pr.nibble(6) << 4;  // leaves of the patch
+#pragma unroll 1
+  for (int s = 0; s < 2; ++s) {
+    const bool active = s ? two : any;
+    const unsigned mask = __ballot_sync(0xffffffffu, active);
+    if (!active) continue;
+    uint32_t o[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) o[j] = s ? o1[j] : o0[j];
+    auto at = [&](const float* base, int a) {
+      const uint32_t off = a & 1 ? o[a >> 1] >> 16 : o[a >> 1] & 0xffffu;
+      return *reinterpret_cast<const float*>(reinterpret_cast<const char*>(base) + off);
+    };
+    float r[Op::NC][8];
+    Op::leaf(cst[s ? l1 : l0], k, xs, fs, at, qd + (s ? n1 : n0), ne, r);
+#pragma unroll
+    for (int a = 0; a < 8; ++a) {
+      const uint32_t off = a & 1 ? o[a >> 1] >> 16 : o[a >> 1] & 0xffffu;
+      char* p = reinterpret_cast<char*>(yw) + off;
+      __syncwarp(mask);
+      float t[Op::NC];
+#pragma unroll
+      for (int n = 0; n < Op::NC; ++n)
+        t[n] = *reinterpret_cast<volatile float*>(p + n * kPatchSlots * 4);
+#pragma unroll
+      for (int n = 0; n < Op::NC; ++n)
+        *reinterpret_cast<volatile float*>(p + n * kPatchSlots * 4) = t[n] + r[n][a];
+    }
+    __syncwarp(mask);
+  }
+}
 
 template <class Op, class C, bool CGP>
 __global__ void __launch_bounds__(kTileThreads, Op::CTAS)
 k_apply_tile(MeshDev m, DevParams p, CoefArgs<C> cf, const float* __restrict__ x,
              float* __restrict__ y, double* __restrict__ S_cg, int par, int fcg,
              const float* __restrict__ zcg, float* __restrict__ pout) {
-  constexpr int NC = Op::NC, NA = NC + (CGP ? 1 : 0) + (Op::FIELD ? 1 : 0);
+  constexpr int NC = Op::NC, NF = Op::NF, F0 = NC + (CGP ? 1 : 0), NA = F0 + NF;
   constexpr int kWarps = kTileThreads / 32;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float* ys = reinterpret_cast<float*>(smem_raw);   // [warps][NC][kPatchSlots] sums
   float* xb = ys + kWarps * NC * kPatchSlots;                      // [NC][kPatchSlots] node values
-  float* fs = xb + NC * kPatchSlots;                // s = 1 + phi~ per slot (FIELD)
+  float* fs = xb + NC * kPatchSlots;                // [NF][kPatchSlots] fields
   __shared__ float4 s_cst[CHNS_MAXD];
   __shared__ float s_beta;
   const int tid = threadIdx.x, G = gridDim.x;
   const int np = (int)m.n_patch, N = (int)m.n_nodes;
   const PrmT<float>& k = p.f;
-  const float shift = 1.f + cf.phi_shift;
+  const float shift = (Op::ONE_PLUS ? 1.f : 0.f) + cf.phi_shift;
   if (CGP && tid == 0) {
     // CG direction update fused into the gather: p_new = z + beta p_old with
     // beta = rz_cur / rz_prev (fcg: Polak-Ribiere)
@@ -439,7 +605,9 @@ k_apply_tile(MeshDev m, DevParams p, CoefArgs<C> cf, const float* __restrict__ x
 #pragma unroll
     for (int c = 0; c < NC; ++c) v[c] = __ldg(x + (int64_t)c * N + g);
     if (CGP) v[NC] = __ldg(zcg + g);
-    if (Op::FIELD) v[NA - 1] = ldv<float>(cf.phi, g);
+    if constexpr (NF > 0) v[F0] = ldv<float>(cf.phi, g);
+#pragma unroll
+    for (int f = 1; f < NF; ++f) v[F0 + f] = ldv<float>(f < 4 ? cf.u[f - 1] : cf.mu, g);
   };
   auto load_ids = [&](const uint4& h, uint32_t id[kPreSlots]) {
     const int last = (int)(h.y & 0xffffu) - 1;
@@ -479,12 +647,13 @@ k_apply_tile(MeshDev m, DevParams p, CoefArgs<C> cf, const float* __restrict__ x
   uint4 h = head_of(t), h1 = head_of(t + G);
   TilePre<NA> q;
   load_ids(h, q.id);
-  load_rest(h, q);
+  if (Op::AHEAD) load_rest(h, q);
   if (CGP) __syncthreads();
   const float beta = CGP ? s_beta : 0.f;
   for (; t < np; t += G) {
     const int nreg = (int)(h.y & 0xffffu), nhang = (int)(h.y >> 16);
     const int nb4 = 4 * (int)(h.z & 0xffffu), nt = nb4 + (((int)(h.z >> 16) + 1) >> 1);
+    if (!Op::AHEAD) load_rest(h, q);
     // 1. node values to shared memory
     auto put = [&](int i, uint32_t id, const float v[NA]) {
       const int g = (int)(id & kNodeMask);
@@ -499,7 +668,8 @@ k_apply_tile(MeshDev m, DevParams p, CoefArgs<C> cf, const float* __restrict__ x
         if (dir) y[(int64_t)c * N + g] = xv;  // identity rows, likewise
         xb[c * kPatchSlots + i] = dir ? 0.f : xv;
       }
-      if (Op::FIELD) fs[i] = v[NA - 1] + shift;
+#pragma unroll
+      for (int f = 0; f < NF; ++f) fs[f * kPatchSlots + i] = f == 0 ? v[F0] + shift : v[F0 + f];
     };
 #pragma unroll
     for (int u = 0; u < kPreSlots; ++u)
@@ -524,42 +694,51 @@ k_apply_tile(MeshDev m, DevParams p, CoefArgs<C> cf, const float* __restrict__ x
           float* v = xb + n * kPatchSlots;
           v[nreg + i] = 0.25f * ((v[a] + v[b]) + (v[c] + v[d]));
         }
-        if (Op::FIELD) fs[nreg + i] = 0.25f * ((fs[a] + fs[b]) + (fs[c] + fs[d]));
+#pragma unroll
+        for (int f = 0; f < NF; ++f) {
+          float* v = fs + f * kPatchSlots;
+          v[nreg + i] = 0.25f * ((v[a] + v[b]) + (v[c] + v[d]));
+        }
       }
       __syncthreads();
     }
     // 2.-3. elements
-    const unsigned mask_b = __ballot_sync(0xffffffffu, tid < nb4);
-    const unsigned mask_s = __ballot_sync(0xffffffffu, tid >= nb4 && tid < nt);
     float* yw = ys + (tid >> 5) * NC * kPatchSlots;
-    if (tid < nt) {
-      F2 r[NC][4][2];
-      Op op;
-      PairConst pc;
-      F2 e(0.f);
-      const uint32_t base = h.w & 0xffffu;
-      if (tid < nb4) {
-        const PairRefs<true> pr{q.ref};
-        const float4 c = s_cst[base + pr.nibble(0)];
-        pc.c[0] = F2(c.x); pc.c[1] = F2(c.y); pc.c[2] = F2(c.z); pc.c[3] = F2(c.w);
-        op.setup(pr, fs, pc, k);
+    if constexpr (Op::FORM == TileForm::kLeaf) {
+      tile_leaves<Op>(k, q.ref, s_cst + (h.w & 0xffffu), tid < nb4, tid < nt, xb, fs,
+                      static_cast<const float*>(cf.qd) + m.patch_elem[t], m.n_elem, yw);
+    } else {
+      const unsigned mask_b = __ballot_sync(0xffffffffu, tid < nb4);
+      const unsigned mask_s = __ballot_sync(0xffffffffu, tid >= nb4 && tid < nt);
+      if (tid < nt) {
+        F2 r[NC][4][2];
+        Op op;
+        PairConst pc;
+        F2 e(0.f);
+        const uint32_t base = h.w & 0xffffu;
+        if (tid < nb4) {
+          const PairRefs<true> pr{q.ref};
+          const float4 c = s_cst[base + pr.nibble(0)];
+          pc.c[0] = F2(c.x); pc.c[1] = F2(c.y); pc.c[2] = F2(c.z); pc.c[3] = F2(c.w);
+          op.setup(pr, fs, pc, k);
 #pragma unroll
-        for (int n = 0; n < NC; ++n) op.apply(k, pr, xb + n * kPatchSlots, r[n], &e);
-        pr.template store<NC>(r, yw, mask_b, true);
-      } else {
-        const PairRefs<false> pr{q.ref};
-        const float4 c = s_cst[base + pr.nibble(0)], d = s_cst[base + pr.nibble(4)];
-        pc.c[0] = F2(c.x, d.x); pc.c[1] = F2(c.y, d.y); pc.c[2] = F2(c.z, d.z); pc.c[3] = F2(c.w, d.w);
-        const bool two = pr.nibble(3) != 0;
-        op.setup(pr, fs, pc, k);
+          for (int n = 0; n < NC; ++n) op.apply(k, pr, xb + n * kPatchSlots, r[n], &e);
+          pr.template store<NC>(r, yw, mask_b, true);
+        } else {
+          const PairRefs<false> pr{q.ref};
+          const float4 c = s_cst[base + pr.nibble(0)], d = s_cst[base + pr.nibble(4)];
+          pc.c[0] = F2(c.x, d.x); pc.c[1] = F2(c.y, d.y); pc.c[2] = F2(c.z, d.z); pc.c[3] = F2(c.w, d.w);
+          const bool two = pr.nibble(3) != 0;
+          op.setup(pr, fs, pc, k);
 #pragma unroll
-        for (int n = 0; n < NC; ++n) op.apply(k, pr, xb + n * kPatchSlots, r[n], &e);
-        pr.template store<NC>(r, yw, mask_s, two);
-        if (!two) e.y = 0.f;
-      }
-      if (Op::ENERGY) {
-        df_addf(en[0], e.x);
-        df_addf(en[0], e.y);
+          for (int n = 0; n < NC; ++n) op.apply(k, pr, xb + n * kPatchSlots, r[n], &e);
+          pr.template store<NC>(r, yw, mask_s, two);
+          if (!two) e.y = 0.f;
+        }
+        if (Op::ENERGY) {
+          df_addf(en[0], e.x);
+          df_addf(en[0], e.y);
+        }
       }
     }
     __syncthreads();
@@ -573,7 +752,7 @@ k_apply_tile(MeshDev m, DevParams p, CoefArgs<C> cf, const float* __restrict__ x
     }
 #pragma unroll
     for (int u = 0; u < kPreHang; ++u) par0[u] = q.par[u];
-    load_rest(h1, q);
+    if (Op::AHEAD) load_rest(h1, q);
     // the sum of slot i over the warps, cleared for the next patch
     auto take = [&](int n, int i) {
       float t[kWarps], v = 0.f;
