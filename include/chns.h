@@ -168,11 +168,11 @@ void chns_mesh_destroy(chns_mesh* mesh);
  *   CHNS_APPLY_STREAM: persistent CTAs, each walking the patches blockIdx, blockIdx + grid, ...
  *                      with two leaves per thread (for the Poisson and mass applies with the next
  *                      patch's node values loaded while the current patch is computed). Used by
- *                      the FP32 Poisson, mass and momentum applies, with FP32 or bfloat16
- *                      coefficients (including the Poisson apply fused into CG); the CH apply
- *                      and the other precisions keep CHNS_APPLY_PATCH.
+ *                      the FP32 applies, with FP32 or bfloat16 coefficients (including the
+ *                      Poisson apply fused into CG); the other precisions keep
+ *                      CHNS_APPLY_PATCH.
  *   CHNS_APPLY_AUTO:   CHNS_APPLY_STREAM where it is the faster one: the Poisson and mass applies
- *                      from 8 patches per SM on, momentum on every mesh.
+ *                      from 8 patches per SM on, CH from 12, momentum on every mesh.
  * max_ctas bounds the persistent grid (0: as many CTAs as the device holds at once). Errors:
  * EINVAL for a null mesh, an unknown kernel or max_ctas < 0. Not thread-safe against applies
  * running on the same mesh from other host threads. */

@@ -272,13 +272,16 @@ static void launch_tile(const chns_mesh* m, const DevParams& p, const CoefArgs<C
 // a CUDA graph, Poisson, per-patch / this: 2,878 leaves 5.9 / 6.6 us, 77,932 7.1 / 7.5, 156,640
 // 8.4 / 8.5, 314,672 (8.2 patches per SM) 13.4 / 12.5, 1,429,744 40.4 / 34.6).
 constexpr int kTilePatchesPerSm = 8;
-// The momentum apply is faster in it on every mesh (see TileMom).
+// The CH apply gains from more patches per SM on (per-patch / this: 314,672 leaves 20.7 / 21.4 us,
+// 525,960 (13.9 patches per SM) 31.3 / 29.4, 756,064 41.0 / 38.9, 1,429,744 85.8 / 72.1); the momentum
+// apply on every mesh (see TileMom).
+constexpr int kTilePatchesPerSmCh = 12;
 template <class T, class S>
 static bool use_tile(const chns_mesh* m, chns_operator op) {
   if (!(std::is_same<T, float>::value && std::is_same<S, float>::value)) return false;
   if (m->apply_kernel == CHNS_APPLY_PATCH) return false;
   if (m->apply_kernel == CHNS_APPLY_STREAM) return true;
-  const int from = op == CHNS_OP_MOMENTUM ? 0 : kTilePatchesPerSm;
+  const int from = op == CHNS_OP_MOMENTUM ? 0 : op == CHNS_OP_CH ? kTilePatchesPerSmCh : kTilePatchesPerSm;
   return m->d.n_patch >= (int64_t)from * std::max(m->sm_count, 1);
 }
 
@@ -437,6 +440,12 @@ static void launch_apply(const chns_mesh* m, chns_operator op, const DevParams& 
       launch_patch<MassK<T, C>, T, S, C, false>(m, p, cf, x, y, nullptr, s);
       break;
     case CHNS_OP_CH:
+      if constexpr (std::is_same<T, float>::value && std::is_same<S, T>::value) {
+        if (use_tile<T, S>(m, op)) {
+          launch_tile<TileCh, C, false>(m, p, cf, x, y, nullptr, s);
+          break;
+        }
+      }
       launch_patch<ChK<T, C>, T, S, C, false>(m, p, cf, x, y, nullptr, s);
       break;
     case CHNS_OP_MOMENTUM: {

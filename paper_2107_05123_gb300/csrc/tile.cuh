@@ -6,7 +6,7 @@
 //  1. the values of the regular slots go to shared memory, then the hanging slots are
 //     interpolated (mean of 2 or 4 parents);
 //  2. each thread applies the element operator to its two leaves, sum-factorised, in packed FP32 pairs
-//     (one issue slot for two operations): Poisson, mass and shifted to both leaves at once,
+//     (one issue slot for two operations): Poisson, mass and shifted to both leaves at once, CH and
 //     momentum to one after the other with pairs of Gauss points;
 //  3. the contributions are added to sums per slot in shared memory, one array per warp, by plain
 //     read-add-write: the threads of a warp add the same corner of their leaves in the same step,
@@ -405,6 +405,113 @@ __device__ __forceinline__ Geo<float> leaf_geometry(const float4& c) {
   g.ih[2] = c.w;
   return g;
 }
+
+// Kron in pairs along x: B, C = Dy Pz u at y = 0 [z], E = Py Dz u at z = 0 [y]
+struct KronP {
+  F2 B[4], C[2], E[2];
+  __device__ __forceinline__ void eval(const float u[8]) {
+    F2 l[4], p[4], w[2];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) l[j] = F2(u[2 * j], u[2 * j + 1]);
+#pragma unroll
+    for (int y = 0; y < 2; ++y) {
+      p[y] = mad(F2(2.f), l[y], l[y + 2]);
+      p[y + 2] = mad(F2(2.f), l[y + 2], l[y]);
+      w[y] = l[y] - l[y + 2];
+    }
+#pragma unroll
+    for (int z = 0; z < 2; ++z) {
+      B[2 * z] = mad(F2(2.f), p[2 * z], p[2 * z + 1]);
+      B[2 * z + 1] = mad(F2(2.f), p[2 * z + 1], p[2 * z]);
+      C[z] = p[2 * z] - p[2 * z + 1];
+    }
+    E[0] = mad(F2(2.f), w[0], w[1]);
+    E[1] = mad(F2(2.f), w[1], w[0]);
+  }
+  // r = Px (cm B + c (kh_y C' + kh_z E')) + c kh_x Dx B' with the stiffness part of field o
+  __device__ __forceinline__ void sum(float cm, const KronP& o, float c, const float kh[3],
+                                      F2 r[4]) const {
+    const F2 cy(c * kh[1]), cz(c * kh[2]);
+    const float cx = c * kh[0];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const F2 yc = j & 1 ? -o.C[j >> 1] : o.C[j >> 1], ze = j & 2 ? -o.E[j & 1] : o.E[j & 1];
+      const F2 S = mad(F2(cm), B[j], mad(cy, yc, cz * ze));
+      const float d = cx * (o.B[j].x - o.B[j].y);
+      r[j] = F2(fmaf(2.f, S.x, S.y) + d, fmaf(2.f, S.y, S.x) - d);
+    }
+  }
+};
+
+// The Cahn-Hilliard Jacobian (see ChK) in (dphi, dmu), one leaf after the other in packed pairs
+// along x. Bound by latency (31 % of the issue slots with both leaves at once): five CTAs per SM at 96
+// registers. FP32 on 1,429,744 leaves, in a CUDA graph: 72.1 us, CTA-per-patch kernel 85.8, both
+// leaves at once in packed pairs 76.8 (four CTAs, 128 registers) and 81.4 (three, 149); six CTAs
+// 81.0 (108 bytes of spills), the next patch's values loaded ahead 73.1.
+struct TileCh {
+  static constexpr int NC = 2;
+  static constexpr int NF = 4;  // phi~, u~
+  static constexpr bool ONE_PLUS = false, AHEAD = false, DIR = false, ENERGY = false;
+  static constexpr TileForm FORM = TileForm::kLeaf;
+  static constexpr int CTAS = 5;
+  static __device__ __forceinline__ float4 consts(const LevelGeo& g, const PrmT<float>&) {
+    return leaf_consts(g);
+  }
+  template <class At>
+  static __device__ __forceinline__ void leaf(const float4& c, const PrmT<float>& k, const float* xs,
+                                              const float* fs, const At& at, const float*, int64_t,
+                                              float (&r)[NC][8]) {
+    constexpr double w = gauss_w<float>(), w3 = w * w * w;
+    const Geo<float> g = leaf_geometry(c);
+    const float J = g.detJ, *ih = g.ih;
+    F2 R[2][4], fv[4], t[4], o[4];
+    float v[8];
+    auto get = [&](const float* base) {
+#pragma unroll
+      for (int a = 0; a < 8; ++a) v[a] = at(base, a);
+    };
+    get(xs);
+    interp3<false>(v, fv);
+    {
+      const float cm = J * (float)(8.0 / 216.0), ks = J * (float)(8.0 / 36.0);
+      const float kh[3] = {ks * ih[0] * ih[0], ks * ih[1] * ih[1], ks * ih[2] * ih[2]};
+      KronP f, m;
+      f.eval(v);
+      get(xs + kPatchSlots);
+      m.eval(v);
+      f.sum(cm * k.idt, m, k.kmu, kh, R[0]);
+      m.sum(-0.5f * cm, f, k.kphi, kh, R[1]);
+    }
+    // 1/2 (q, psi''(phi~) dphi), psi'' = 3 phi~^2 - 1
+    get(fs);
+    interp3<false>(v, t);
+    const F2 cs((float)(0.5 * w3 * w3) * J), c3 = cs * F2((float)(3.0 * w3 * w3));
+#pragma unroll
+    for (int j = 0; j < 4; ++j) t[j] = mad(c3 * t[j], t[j], -cs) * fv[j];
+    interp3_t<false>(t, o);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) R[1][j] += o[j];
+    // -1/2 (grad q, u~ dphi)
+    GradP d;
+#pragma unroll
+    for (int n = 0; n < 3; ++n) {
+      get(fs + (1 + n) * kPatchSlots);
+      interp3<false>(v, t);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) d.sum(j, n, t[j] * fv[j]);
+    }
+    const float ca = (float)(-0.5 * w3 * w3 * w * w) * J;
+    const float sc[3] = {ca * ih[0], ca * ih[1], ca * ih[2]};
+    d.transpose(sc, R[0]);
+#pragma unroll
+    for (int n = 0; n < 2; ++n)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        r[n][2 * j] = R[n][j].x;
+        r[n][2 * j + 1] = R[n][j].y;
+      }
+  }
+};
 
 // The momentum operator with its coefficients evaluated on the fly (see MomK), one leaf after the
 // other in packed pairs of Gauss points. Bound by latency (as CTA-per-patch kernel: 34 % of the issue
