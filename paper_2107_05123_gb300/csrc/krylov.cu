@@ -416,7 +416,10 @@ void orth_update(const T* V, int64_t ld, int nk, const double* h, T* w, int64_t 
 // the L2 costs: its time is latency, about 10 us for 30 vectors of 36,530.
 constexpr int kArnoldiThreads = 512;
 constexpr int kArnoldiMax = 64;          // restart + 1 sums
-constexpr int kArnoldiSlice = 40 * 1024;  // bytes of w per CTA: longer vectors take the kernels below
+// bytes of w per CTA: longer vectors take the kernels below, whose dot products run in many more CTAs.
+// Momentum solves (3 unknowns per node, FP32), those kernels / this: 38,487 leaves (3 KB) 4.74 / 4.05 ms,
+// 111,504 (9 KB) 6.71 / 6.75, 154,120 (11 KB) 7.52 / 8.60, 321,112 (25 KB) 10.1 / 16.7.
+constexpr int kArnoldiSlice = 6 * 1024;
 
 // Waits until all CTAs of the launch have arrived `round` times; false when it gave up (a limit of
 // about a second: nothing the caller can continue from).
