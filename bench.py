@@ -445,7 +445,7 @@ def run_ours(args):
         "e2e": {"value": e2e_val, "unit": UNIT, "h2d_bytes_per_step": int(2 * N * 8),
                 "d2h_bytes_per_step": int(N * 8)},
         "roofline": None if pa is None else {
-            "kernel": "Poisson apply FP32 (k_apply_stream<PoissonK<float,float>>)", "bound": "hbm",
+            "kernel": "Poisson apply FP32 (k_apply_tile<TilePoisson>)", "bound": "hbm",
             "achieved": pa["achieved_gbs"], "peak": peak, "peak_kind": peak_kind, "unit": "GB/s",
             "frac": pa["frac"], "traffic": traffic, "alg_bytes": pa["alg_bytes"], "ms": pa["ms"]},
         "applies_hbm_frac_fp32": None if not applies else {
