@@ -269,8 +269,10 @@ static void launch_tile(const chns_mesh* m, const DevParams& p, const CoefArgs<C
 // FP32 vectors take the two-leaves-per-thread kernel from kTilePatchesPerSm patches per SM on: its
 // CTAs then have patches to load ahead, while on smaller meshes, where one patch's latency is the
 // whole time, the CTA-per-patch kernel with one leaf per thread is as fast or faster (measured in
-// a CUDA graph, Poisson, per-patch / this: 2,878 leaves 5.9 / 6.6 us, 77,932 7.1 / 7.5, 156,640
-// 8.4 / 8.5, 314,672 (8.2 patches per SM) 13.4 / 12.5, 1,429,744 40.4 / 34.6).
+// a CUDA graph, per-patch / this: Poisson on 19,608 leaves 5.8 / 6.5 us, 77,932 6.7 / 7.1, 156,640
+// 8.1 / 8.2, 314,672 (8.2 patches per SM) 12.9 / 11.8, 635,328 17.7 / 15.6, 1,429,744 38.7 / 32.9; mass
+// on 156,640 14.8 / 14.7, 314,672 24.6 / 23.0, 635,328 33.4 / 35.0, 756,064 40.6 / 40.5, 1,429,744
+// 80.5 / 74.9).
 constexpr int kTilePatchesPerSm = 8;
 // The CH apply gains from more patches per SM on (per-patch / this: 314,672 leaves 20.7 / 21.4 us,
 // 525,960 (13.9 patches per SM) 31.3 / 29.4, 756,064 41.0 / 38.9, 1,429,744 85.8 / 72.1); the momentum

@@ -11,7 +11,9 @@
 //  3. the contributions are added to sums per slot in shared memory, one array per warp, by plain
 //     read-add-write: the threads of a warp add the same corner of their leaves in the same step,
 //     and a point is that corner of at most one leaf (the one that fills that octant around it),
-//     so no two of them meet. The leaves of a brick pair add up their four shared nodes first
+//     so no two of them meet. That holds within the steps of one kind of pair; brick pairs and
+//     others of a warp have different steps and add one kind after the other, with a barrier of
+//     the whole warp in between. The leaves of a brick pair add up their four shared nodes first
 //     (six additions per leaf);
 //  4. the sums of the hanging slots are distributed to their parents with the same weights, and
 //     each regular slot is written once: a plain store where the patch owns the node, a global
@@ -26,11 +28,12 @@
 // stalls), on large meshes also the index records (21 bytes per leaf of 35). Measured against one
 // thread per leaf with shared-memory float atomics (a compare-and-swap loop on this part, 5.3 cycles
 // per warp operation against 2.1 for the read-add-write and 26 against 9.6 in latency): Poisson
-// on 6.9e6 leaves 185 -> 145 us, mass (bfloat16 coefficients) on 3.1e5 32.7 -> 26.7 us with the
+// on 6.9e6 leaves 185 -> 147 us, mass (bfloat16 coefficients) on 3.1e5 32.7 -> 28.0 us with the
 // identity rows' kernel gone. Also measured, slower (Poisson, 6.9e6 leaves): one warp per patch
 // and a lane per brick 190 us (150 registers leave 9 warps per SM); per-slot lists of contributions
 // instead of sums in place 155 us (the lists double the traffic); shared atomics here 174 us; 6
-// or 8 CTAs per SM 153 and 155 us.
+// or 8 CTAs per SM 153 and 155 us. With the elements of both kinds of pair before the sums of either:
+// 1,429,744 leaves, Poisson 32.9 -> 33.8 us and mass 74.9 -> 79.1 us in a CUDA graph.
 #pragma once
 
 #include "ops.cuh"
@@ -815,36 +818,46 @@ k_apply_tile(MeshDev m, DevParams p, CoefArgs<C> cf, const float* __restrict__ x
       tile_leaves<Op>(k, q.ref, s_cst + (h.w & 0xffffu), tid < nb4, tid < nt, xb, fs,
                       static_cast<const float*>(cf.qd) + m.patch_elem[t], m.n_elem, yw);
     } else {
-      const unsigned mask_b = __ballot_sync(0xffffffffu, tid < nb4);
-      const unsigned mask_s = __ballot_sync(0xffffffffu, tid >= nb4 && tid < nt);
-      if (tid < nt) {
+      // brick pairs, then the others: a warp that has both takes them one after the other, with all
+      // its lanes meeting in between, since a slot can be a corner of leaves of either kind
+      const bool brick = tid < nb4, other = tid >= nb4 && tid < nt;
+      const unsigned mask_b = __ballot_sync(0xffffffffu, brick);
+      const unsigned mask_s = __ballot_sync(0xffffffffu, other);
+      const uint32_t base = h.w & 0xffffu;
+      if (brick) {
         F2 r[NC][4][2];
         Op op;
         PairConst pc;
         F2 e(0.f);
-        const uint32_t base = h.w & 0xffffu;
-        if (tid < nb4) {
-          const PairRefs<true> pr{q.ref};
-          const float4 c = s_cst[base + pr.nibble(0)];
-          pc.c[0] = F2(c.x); pc.c[1] = F2(c.y); pc.c[2] = F2(c.z); pc.c[3] = F2(c.w);
-          op.setup(pr, fs, pc, k);
+        const PairRefs<true> pr{q.ref};
+        const float4 c = s_cst[base + pr.nibble(0)];
+        pc.c[0] = F2(c.x); pc.c[1] = F2(c.y); pc.c[2] = F2(c.z); pc.c[3] = F2(c.w);
+        op.setup(pr, fs, pc, k);
 #pragma unroll
-          for (int n = 0; n < NC; ++n) op.apply(k, pr, xb + n * kPatchSlots, r[n], &e);
-          pr.template store<NC>(r, yw, mask_b, true);
-        } else {
-          const PairRefs<false> pr{q.ref};
-          const float4 c = s_cst[base + pr.nibble(0)], d = s_cst[base + pr.nibble(4)];
-          pc.c[0] = F2(c.x, d.x); pc.c[1] = F2(c.y, d.y); pc.c[2] = F2(c.z, d.z); pc.c[3] = F2(c.w, d.w);
-          const bool two = pr.nibble(3) != 0;
-          op.setup(pr, fs, pc, k);
-#pragma unroll
-          for (int n = 0; n < NC; ++n) op.apply(k, pr, xb + n * kPatchSlots, r[n], &e);
-          pr.template store<NC>(r, yw, mask_s, two);
-          if (!two) e.y = 0.f;
-        }
+        for (int n = 0; n < NC; ++n) op.apply(k, pr, xb + n * kPatchSlots, r[n], &e);
+        pr.template store<NC>(r, yw, mask_b, true);
         if (Op::ENERGY) {
           df_addf(en[0], e.x);
           df_addf(en[0], e.y);
+        }
+      }
+      __syncwarp();
+      if (other) {
+        F2 r[NC][4][2];
+        Op op;
+        PairConst pc;
+        F2 e(0.f);
+        const PairRefs<false> pr{q.ref};
+        const float4 c = s_cst[base + pr.nibble(0)], d = s_cst[base + pr.nibble(4)];
+        pc.c[0] = F2(c.x, d.x); pc.c[1] = F2(c.y, d.y); pc.c[2] = F2(c.z, d.z); pc.c[3] = F2(c.w, d.w);
+        const bool two = pr.nibble(3) != 0;
+        op.setup(pr, fs, pc, k);
+#pragma unroll
+        for (int n = 0; n < NC; ++n) op.apply(k, pr, xb + n * kPatchSlots, r[n], &e);
+        pr.template store<NC>(r, yw, mask_s, two);
+        if (Op::ENERGY) {
+          df_addf(en[0], e.x);
+          if (two) df_addf(en[0], e.y);
         }
       }
     }
@@ -912,7 +925,7 @@ k_apply_tile(MeshDev m, DevParams p, CoefArgs<C> cf, const float* __restrict__ x
         write(i, __ldg(rec_of(h) + i));
     h = h1;
     h1 = h2;
-    // (two barriers of the next patch stand between these reads and the next sums)
+    // (a barrier of the next patch stands between these reads and the next sums)
   }
   if (Op::ENERGY) {
     double tot[1];
