@@ -32,6 +32,9 @@ constexpr uint32_t kElocLevelMask = 0x1f;
 // leaves two by two.
 constexpr int kTileThreads = 128;
 static_assert(2 * kTileThreads == kPatchElems && 4 * kPatchSlots <= 0x1000, "references");
+// Levels of a patch above its lowest: a reference holds a leaf's in 4 bits. A chain of leaves refined
+// towards one point spans 19 levels in 134 leaves, so patches are closed by this limit too.
+constexpr int kPatchLevelSpan = 15;
 // Head of a patch: first 16-byte unit of its index record; regular | hanging slots << 16; bricks |
 // other leaves << 16; lowest level | units from the record to its references << 16. Sections of
 // the record (32-bit words, each on a 16-byte boundary):

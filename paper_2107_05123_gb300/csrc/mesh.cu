@@ -156,8 +156,9 @@ void free_mesh(chns_mesh* m) {
 // Greedy partition of the Morton-ordered elements into patches (see kPatchElems/kPatchSlots and
 // the index record in internal.h): regular slots = distinct nodes used as corners or as parents
 // of hanging corners, hanging slots = distinct hanging corners; a node is owned by a patch when no
-// other patch has it as a slot. Bricks are never split. The leaf list is cut into chunks of
-// kPatchChunk leaves (moved to the next unit) that are partitioned in parallel.
+// other patch has it as a slot. Bricks are never split, and the levels of a patch span at most
+// kPatchLevelSpan. The leaf list is cut into chunks of kPatchChunk leaves (moved to the next unit) that
+// are partitioned in parallel.
 struct PatchTables {
   std::vector<int32_t> elem;  // per patch: first element
   std::vector<uint4> head;
@@ -354,14 +355,22 @@ struct PatchBuilder {
     std::vector<std::pair<int32_t, int32_t>> units;
     map.clear();
     int64_t e0 = b;
+    int low = CHNS_MAXD, high = 0;  // levels of the current patch
     for (int64_t i = b; i < e;) {
-      const int n = unit[i];
-      if (i - e0 + n > kPatchElems || !add_unit(i, n, i == e0)) {
+      const int n = unit[i], l = levels[i];
+      if (i > e0 && (i - e0 + n > kPatchElems ||
+                     std::max(high, l) - std::min(low, l) > kPatchLevelSpan ||
+                     !add_unit(i, n, false))) {
         close(e0, i, units);
         units.clear();
         e0 = i;
+        low = CHNS_MAXD;
+        high = 0;
         continue;
       }
+      if (i == e0) add_unit(i, n, true);
+      low = std::min(low, l);
+      high = std::max(high, l);
       units.push_back({(int32_t)i, n});
       i += n;
     }
