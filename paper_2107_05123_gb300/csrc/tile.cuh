@@ -521,7 +521,7 @@ struct TileCh {
 // slots, barriers 25 % and loads of the gather 20 % of the stalls): three CTAs of four warps at 168
 // registers overlap their phases better than two of eight at 128, and the sums need no
 // compare-and-swap loops, 24 per leaf. FP32 in a CUDA graph, CTA-per-patch kernel / this: 1,429,744
-// leaves 217 / 143 us, 314,672 48.0 / 36.5, 77,932 19.6 / 15.6, 19,608 12.6 / 11.8; four CTAs at 128
+// leaves 210 / 148 us, 314,672 46.7 / 37.4, 77,932 19.4 / 15.5, 19,608 12.7 / 12.4; four CTAs at 128
 // registers 194 us on the first (412 bytes of spills), in scalar arithmetic 178 us.
 struct TileMom {
   static constexpr int NC = 3;
