@@ -67,12 +67,12 @@ k_residual_ch(MeshDev m, DevParams p, const double* __restrict__ phi, const doub
     for (int i = 0; i < 8; ++i) s[i] = mad(-cm, kq.B[i], mad(py, kp.c_at(i), pz * kp.e_at(i)));
     kp.finish(s, k.cn2 * kh[0], r1);
   }
+  // phi~ normalised, so that a pure phase (phi = 1 or -1, mu = 0) has no residual, without rounding
   A pv[8];
-  interp3<false>(pt, pv);
-  // (q, phi^3 - phi) from the unnormalised values: w^3 (test) (w^9 p^3 - w^3 p)
-  const A c1 = J * A(w3 * w3), c3 = c1 * A(w3 * w3);
+  interp3<true>(pt, pv);
+  const A c1 = J * A(w3);
 #pragma unroll
-  for (int q = 0; q < 8; ++q) s[q] = mad(c3 * pv[q], pv[q], -c1) * pv[q];
+  for (int q = 0; q < 8; ++q) s[q] = mad(c1 * pv[q], pv[q], -c1) * pv[q];
   A t[8];
   interp3<false>(s, t);
 #pragma unroll
@@ -84,7 +84,7 @@ k_residual_ch(MeshDev m, DevParams p, const double* __restrict__ phi, const doub
 #pragma unroll
     for (int q = 0; q < 8; ++q) d.sum(q, c, t[q] * pv[q]);
   }
-  const A ca = J * A(-w3 * w3 * w * w);
+  const A ca = J * A(-w3 * w * w);
   const A sc[3] = {ca * g.ih[0], ca * g.ih[1], ca * g.ih[2]};
   d.transpose(sc, r0);
   scatter<A, false>(m, idx, r0, f);
