@@ -2,9 +2,10 @@
 // velocity update) and right-preconditioned restarted GMRES (Cahn-Hilliard Newton steps,
 // velocity prediction). The paper solves these systems with PETSc Krylov methods (Appendix A);
 // here every vector update and every dot product is a fused device kernel, dot products and norms
-// are accumulated in FP64 with a deterministic two-level reduction (per-block partial sums, then
-// a fixed-order sum in the last block), and CG keeps its scalars on the device so that the host
-// only reads the residual norm every `check_every` iterations.
+// are accumulated in FP64 (k_dot and the GMRES multi-dot in a fixed order: per-block partial sums,
+// then a sum in the last block or a second kernel; the sums that CG's fused kernels and k_arnoldi
+// form are atomics, in no fixed order), and CG keeps its scalars on the device so that the host only
+// reads the residual norm every `check_every` iterations.
 //
 // Mixed precision: with an FP32 inner precision the Krylov iteration runs on FP32 vectors and FP32
 // (or BF16-coefficient) applies, with FP64 dot products, inside an FP64 iterative-refinement loop
@@ -421,8 +422,8 @@ constexpr int kArnoldiMax = 64;          // restart + 1 sums
 // 111,504 (9 KB) 6.71 / 6.75, 154,120 (11 KB) 7.52 / 8.60, 321,112 (25 KB) 10.1 / 16.7.
 constexpr int kArnoldiSlice = 6 * 1024;
 
-// Waits until all CTAs of the launch have arrived `round` times; false when it gave up (a limit of
-// about a second: nothing the caller can continue from).
+// Waits until all CTAs of the launch have arrived `round` times; false when it gave up, after some
+// seconds (nothing the caller can continue from).
 __device__ __forceinline__ bool grid_arrive_wait(unsigned* bar, unsigned round) {
   __shared__ int ok;
   __syncthreads();
@@ -439,8 +440,8 @@ __device__ __forceinline__ bool grid_arrive_wait(unsigned* bar, unsigned round) 
   return ok;
 }
 
-// acc[k] += sum over the slice of V_k w (k < nk) and w.w (k = nk): one warp per row, four rows at a
-// time so that their loads overlap
+// acc[k] += sum over the slice of V_k w (k < nk) and w.w (k = nk): a warp takes R rows at a time, so
+// that their loads overlap
 template <class T>
 __device__ __forceinline__ void slice_dots(const T* __restrict__ V, int64_t ld, int nk,
                                            const T* ws, int64_t i0, int len, double* acc) {
@@ -1251,18 +1252,25 @@ static double* arnoldi_out(const Ctx& c, int par) {
   return c.m->ws.red + 2 * kRedSlots + (4 + par) * kArnoldiMax;
 }
 
+// *refused: the launch does not fit what this context may use of the device, and did not run
 template <class T>
 chns_status arnoldi(const Ctx& c, const T* V, int64_t ld, int nk, T* w, int64_t n, int chunk,
-                    int par) {
+                    int par, bool* refused) {
   unsigned* bar = reinterpret_cast<unsigned*>(arnoldi_acc(c, 0) + 6 * kArnoldiMax);
   double *acc = arnoldi_acc(c, par), *next = arnoldi_acc(c, par ^ 1), *out = arnoldi_out(c, par);
   unsigned *b0 = bar + 2 * par, *b1 = bar + 2 * (par ^ 1);
   void* args[] = {(void*)&V, (void*)&ld, (void*)&nk,   (void*)&w,  (void*)&n, (void*)&chunk,
                   (void*)&acc, (void*)&next, (void*)&b0, (void*)&b1, (void*)&out};
+  const cudaError_t e =
+      cudaLaunchCooperativeKernel((const void*)k_arnoldi<T>, dim3((unsigned)c.m->sm_count),
+                                  dim3(kArnoldiThreads), args, (size_t)chunk * sizeof(T), c.s);
+  *refused = e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported;
+  if (*refused) {
+    cudaGetLastError();
+    return CHNS_OK;
+  }
   note_launch();
-  CHNS_CUDA(cudaLaunchCooperativeKernel((const void*)k_arnoldi<T>, dim3((unsigned)c.m->sm_count),
-                                        dim3(kArnoldiThreads), args, (size_t)chunk * sizeof(T),
-                                        c.s));
+  if (e != cudaSuccess) return cuda_fail(e, "cudaLaunchCooperativeKernel");
   return CHNS_OK;
 }
 
@@ -1288,7 +1296,7 @@ chns_status gmres(const Ctx& c, const T* b, T* x, const T* dinv, bool block2, do
   chns_status st;
   // slices of k_arnoldi: one CTA per SM
   const int64_t chunk = (n + c.m->sm_count - 1) / std::max(c.m->sm_count, 1);
-  const bool fused = chunk * (int64_t)sizeof(T) <= kArnoldiSlice;
+  bool fused = chunk * (int64_t)sizeof(T) <= kArnoldiSlice;
   struct Events {
     cudaEvent_t e[2] = {nullptr, nullptr};
     ~Events() {
@@ -1376,8 +1384,19 @@ chns_status gmres(const Ctx& c, const T* b, T* x, const T* dinv, bool block2, do
       if (st != CHNS_OK) return st;
       const int nk = j + 1;
       if (fused) {
-        st = arnoldi<T>(c, V, ld, nk, w, n, (int)chunk, j & 1);
+        bool refused = false;
+        st = arnoldi<T>(c, V, ld, nk, w, n, (int)chunk, j & 1, &refused);
         if (st != CHNS_OK) return st;
+        if (refused) {  // the separate kernels from here on, after the column still in flight
+          fused = false;
+          if (!spc && j > 0) {
+            st = fused_column(j - 1);
+            if (st != CHNS_OK) return st;
+            if (stop) break;
+          }
+        }
+      }
+      if (fused) {
         CHNS_CUDA(cudaMemcpyAsync(c.m->ws.h_pinned + kArnoldiPinned + (j & 1) * kArnoldiMax,
                                   arnoldi_out(c, j & 1), (nk + 1) * sizeof(double),
                                   cudaMemcpyDeviceToHost, c.s));
