@@ -411,12 +411,13 @@ void orth_update(const T* V, int64_t ld, int nk, const double* h, T* w, int64_t 
 // half its norm to the projection a second pass, then w normalised. out[k] = the column of the
 // Hessenberg matrix (k < nk), out[nk] = the norm of the new vector before it was normalised.
 // Each CTA keeps its slice of w in shared memory. Sums over the CTAs are FP64 atomics into acc
-// (two rows of kArnoldiMax, zero on entry; acc_next is cleared for the next step). Against the
+// (two rows of kArnoldiMax, zero on entry; acc_next is cleared for the next step). A CTA whose wait
+// runs out sets out[kArnoldiMax - 1] (zero on entry), which the host reads. Against the
 // separate kernels (multi-dot, final sum, update, each twice, and a host decision between them) it
 // saves five launches and a synchronisation per GMRES iteration, which is what a basis that fits
 // the L2 costs: its time is latency, about 10 us for 30 vectors of 36,530.
 constexpr int kArnoldiThreads = 512;
-constexpr int kArnoldiMax = 64;          // restart + 1 sums
+constexpr int kArnoldiMax = 64;          // restart + 1 sums and the mark of a wait that ran out
 // bytes of w per CTA: longer vectors take the kernels below, whose dot products run in many more CTAs.
 // Momentum solves (3 unknowns per node, FP32), those kernels / this: 38,487 leaves (3 KB) 4.74 / 4.05 ms,
 // 111,504 (9 KB) 6.71 / 6.75, 154,120 (11 KB) 7.52 / 8.60, 321,112 (25 KB) 10.1 / 16.7.
@@ -537,9 +538,9 @@ k_arnoldi(const T* __restrict__ V, int64_t ld, int nk, T* __restrict__ w, int64_
   for (int i = threadIdx.x; i < len; i += kArnoldiThreads) w[i0 + i] = ws[i] * sc;
   if (blockIdx.x == 0) {
     if (threadIdx.x < nk) out[threadIdx.x] = h1;
-    // a NaN norm stops the solve (as does a barrier that gave up)
-    if (threadIdx.x == 0) out[nk] = !ok ? nan("") : nn > 0.0 ? sqrt(nn) : nn == nn ? 0.0 : nn;
+    if (threadIdx.x == 0) out[nk] = nn > 0.0 ? sqrt(nn) : nn == nn ? 0.0 : nn;  // (NaN stays)
   }
+  if (!ok && threadIdx.x == 0) out[kArnoldiMax - 1] = 1.0;
 }
 
 template <class T>
@@ -1242,7 +1243,7 @@ unsigned multidot(const chns_mesh* m, const T* V, int64_t ld, int nk, const T* w
 // [2][kArnoldiMax], barriers [2]
 constexpr int kArnoldiPinned = 128;  // offset in the pinned scalars
 constexpr size_t kArnoldiBytes = (6 * kArnoldiMax + 2) * sizeof(double);
-static_assert(6 * kArnoldiMax + 2 <= kRedSlots && CHNS_GMRES_MAX_RESTART + 1 <= kArnoldiMax &&
+static_assert(6 * kArnoldiMax + 2 <= kRedSlots && CHNS_GMRES_MAX_RESTART + 1 < kArnoldiMax &&
                   kArnoldiPinned + 2 * kArnoldiMax <= 1024,
               "k_arnoldi scratch");
 static double* arnoldi_acc(const Ctx& c, int par) {
@@ -1363,6 +1364,11 @@ chns_status gmres(const Ctx& c, const T* b, T* x, const T* dinv, bool block2, do
     auto fused_column = [&](int j) -> chns_status {
       CHNS_CUDA(cudaEventSynchronize(ev.e[j & 1]));
       const volatile double* o = c.m->ws.h_pinned + kArnoldiPinned + (j & 1) * kArnoldiMax;
+      if (o[kArnoldiMax - 1] != 0.0) {
+        set_error("krylov: a grid barrier of the GMRES Gram-Schmidt kernel timed out");
+        *iters = it;
+        return CHNS_ECUDA;
+      }
       for (int i = 0; i <= j; ++i) Hij(i, j) = o[i];
       return column(j, o[j + 1]);
     };
@@ -1398,7 +1404,7 @@ chns_status gmres(const Ctx& c, const T* b, T* x, const T* dinv, bool block2, do
       }
       if (fused) {
         CHNS_CUDA(cudaMemcpyAsync(c.m->ws.h_pinned + kArnoldiPinned + (j & 1) * kArnoldiMax,
-                                  arnoldi_out(c, j & 1), (nk + 1) * sizeof(double),
+                                  arnoldi_out(c, j & 1), kArnoldiMax * sizeof(double),
                                   cudaMemcpyDeviceToHost, c.s));
         CHNS_CUDA(cudaEventRecord(ev.e[j & 1], c.s));
         if (spc) {

@@ -1,6 +1,7 @@
 """GMRES where the one-launch Gram-Schmidt step cannot run: a context that may use less of the device
 refuses its cooperative launch (from the first one on, or from a later one, with a column still in
-flight). The library is linked with a stand-in for the launch call that returns the refusal.
+flight), and a grid barrier that timed out. The library is linked with a stand-in for the launch call
+that returns the refusal, or sets the mark that a CTA sets whose wait ran out.
 
 The refused solve takes the separate kernels: the iterations and the iterate of the ordinary one,
 1e-9 as between GMRES and its restatement on the host (test_gpu_gmres_restart.py)."""
@@ -23,12 +24,17 @@ from paper_2107_05123_gb300.session import Mesh  # noqa: E402
 FAKE = r"""
 #include <cuda_runtime.h>
 extern "C" {
-int fake_refuse_from = -1, fake_calls = 0;
+int fake_refuse_from = -1, fake_timeout_at = -1, fake_calls = 0;
 cudaError_t fake_cooperative_launch(const void* f, dim3 grid, dim3 block, void** args, size_t smem,
                                     cudaStream_t s) {
   const int call = fake_calls++;
   if (fake_refuse_from >= 0 && call >= fake_refuse_from) return cudaErrorCooperativeLaunchTooLarge;
-  return cudaLaunchCooperativeKernel(f, grid, block, args, smem, s);
+  const cudaError_t e = cudaLaunchCooperativeKernel(f, grid, block, args, smem, s);
+  if (e == cudaSuccess && call == fake_timeout_at) {
+    double* out = *static_cast<double**>(args[10]);
+    return cudaMemsetAsync(out + 63, 1, sizeof(double), s);
+  }
+  return e;
 }
 }
 """
@@ -59,9 +65,9 @@ def lib(tmp_path_factory):
         _lib.LIB_PATH = path
 
 
-def _solve(lib, monkeypatch, restart, its, refuse=-1):
+def _solve(lib, monkeypatch, restart, its, refuse=-1, timeout=-1, check=False):
     monkeypatch.setattr(_lib, "LIB", lib)
-    for name, v in (("fake_refuse_from", refuse), ("fake_calls", 0)):
+    for name, v in (("fake_refuse_from", refuse), ("fake_timeout_at", timeout), ("fake_calls", 0)):
         ctypes.c_int.in_dll(lib, name).value = v
     leaves, ext = LEAVES["drop_l3_5"]
     gm = Mesh(*leaves(), ext)
@@ -71,7 +77,7 @@ def _solve(lib, monkeypatch, restart, its, refuse=-1):
     s = capi.make_solver(capi.KSP_GMRES, capi.PC_JACOBI, 1e-30, its, restart)
     try:
         st = capi.chns_krylov_solve(gm.handle, capi.OP_MOMENTUM, capi.make_params(dict(PRM, dt=5e-2)),
-                                    coef, dev(f["x"].ravel()), x, s, check=False)
+                                    coef, dev(f["x"].ravel()), x, s, check=check)
         return st, x.cpu().numpy(), ctypes.c_int.in_dll(lib, "fake_calls").value
     finally:
         gm.close()
@@ -86,3 +92,10 @@ def test_refused_launch(lib, monkeypatch, restart, its, refuse):
     assert calls2 == refuse + 1  # the first refusal is the last launch tried
     assert st2.iterations == its and st2.status == st.status
     assert relerr(x2, x) < 1e-9
+
+
+@pytest.mark.parametrize("at", [0, 3])
+def test_barrier_timeout_is_reported_as_such(lib, monkeypatch, at):
+    with pytest.raises(_lib.ChnsError, match="timed out") as e:
+        _solve(lib, monkeypatch, 30, 9, timeout=at, check=True)
+    assert e.value.status == capi.ECUDA
