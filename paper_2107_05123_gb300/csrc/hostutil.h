@@ -4,6 +4,7 @@
 
 #include <algorithm>
 #include <cstdint>
+#include <exception>
 #include <thread>
 #include <vector>
 
@@ -41,19 +42,41 @@ inline int threads_for(int64_t n) {
   const int nt = (int)std::max(1u, std::min(16u, std::thread::hardware_concurrency()));
   return (int)std::max<int64_t>(1, std::min<int64_t>(nt, n / 4096));
 }
+// The last part runs on the calling thread, and so does a part whose thread cannot be started; the
+// first part's exception, if any, is thrown again after all have ended.
 template <class F>
 void parallel_parts(int64_t n, int nt, F f) {
-  std::vector<std::thread> th;
   const int64_t chunk = (n + nt - 1) / nt;
-  for (int t = 0; t < nt; ++t) {
-    const int64_t b = t * chunk, e = std::min(n, b + chunk);
-    if (b >= e) break;
-    if (e == n)
-      f(t, b, e);
-    else
-      th.emplace_back([=, &f]() { f(t, b, e); });
+  std::vector<std::exception_ptr> err((size_t)nt);
+  auto run = [&](int t) noexcept {
+    try {
+      f(t, t * chunk, std::min(n, (t + 1) * chunk));
+    } catch (...) {
+      err[(size_t)t] = std::current_exception();
+    }
+  };
+  {
+    struct Threads {
+      std::vector<std::thread> th;
+      ~Threads() {
+        for (auto& t : th) t.join();
+      }
+    } threads;
+    threads.th.reserve((size_t)nt);
+    for (int t = 0; t * chunk < n; ++t) {
+      if ((t + 1) * chunk >= n) {
+        run(t);
+        break;
+      }
+      try {
+        threads.th.emplace_back(run, t);
+      } catch (const std::exception&) {
+        run(t);
+      }
+    }
   }
-  for (auto& t : th) t.join();
+  for (auto& e : err)
+    if (e) std::rethrow_exception(e);
 }
 // Run f(begin, end) over [0, n) on up to 16 threads.
 template <class F>

@@ -406,21 +406,13 @@ static void build_patches(int64_t n, int64_t N, const uint32_t* anchors,
   const int nc = (int)cut.size() - 1;
   std::vector<std::unique_ptr<PatchBuilder>> part(nc);
   std::atomic<int> next(0);
-  std::atomic<bool> failed(false);
-  auto work = [&] {
-    for (int c; (c = next.fetch_add(1)) < nc;) try {
-        part[c].reset(new PatchBuilder{N, enode, hang, levels, unit, P.eloc});
-        part[c]->run(cut[c], cut[c + 1]);
-      } catch (const std::bad_alloc&) {  // no exception leaves a thread
-        failed.store(true);
-      }
-  };
-  const int nt = (int)std::max(1u, std::min(16u, std::thread::hardware_concurrency()));
-  std::vector<std::thread> th;
-  for (int t = 1; t < std::min(nt, nc); ++t) th.emplace_back(work);
-  work();
-  for (auto& t : th) t.join();
-  if (failed.load()) throw std::bad_alloc();
+  const int nt = std::min(nc, (int)std::max(1u, std::min(16u, std::thread::hardware_concurrency())));
+  host::parallel_parts(nt, nt, [&](int, int64_t, int64_t) {
+    for (int c; (c = next.fetch_add(1)) < nc;) {
+      part[c].reset(new PatchBuilder{N, enode, hang, levels, unit, P.eloc});
+      part[c]->run(cut[c], cut[c + 1]);
+    }
+  });
   // concatenate; a node is owned by the only patch that has it as a regular slot
   std::vector<uint8_t> count((size_t)N, 0);
   for (auto& p : part) {
@@ -515,9 +507,7 @@ chns_status build_mesh(const uint32_t* anchors, const uint8_t* levels, int64_t n
   {
     const int nt = host::threads_for(n);
     std::vector<std::vector<uint64_t>> extra(nt);
-    std::atomic<bool> failed(false);
     host::parallel_parts(n, nt, [&](int t, int64_t b, int64_t e) {
-     try {
       for (int64_t i = b; i < e; ++i) {
         uint64_t s = kFull >> levels[i];
         for (int c = 0; c < 8; ++c) {
@@ -534,11 +524,7 @@ chns_status build_mesh(const uint32_t* anchors, const uint8_t* levels, int64_t n
       }
       std::sort(extra[t].begin(), extra[t].end());
       extra[t].erase(std::unique(extra[t].begin(), extra[t].end()), extra[t].end());
-     } catch (const std::bad_alloc&) {  // no exception leaves a thread
-       failed.store(true);
-     }
     });
-    if (failed.load()) throw std::bad_alloc();
     std::vector<uint64_t> all;
     for (auto& v : extra) {
       std::vector<uint64_t> m;
