@@ -451,31 +451,21 @@ static void launch_apply(const chns_mesh* m, chns_operator op, const DevParams& 
       launch_patch<ChK<T, C>, T, S, C, false>(m, p, cf, x, y, nullptr, s);
       break;
     case CHNS_OP_MOMENTUM: {
-      // quadrature data of the running momentum solve, when it matches this precision
-      const void* qd = sizeof(T) == sizeof(double) ? m->mq.qd64 : m->mq.qd32;
-      if (m->mq.on && qd) {
-        CoefArgs<C> cq = cf;
-        cq.qd = qd;
-        if constexpr (std::is_same<T, float>::value && std::is_same<S, T>::value) {
-          // With FP32 coefficients the data hold what the apply itself evaluates, which is faster than
-          // reading 352 bytes per leaf (momentum solve on 321,112 leaves 16.7 ms against 19.0);
-          // bfloat16 coefficients are less accurate than the data (made from FP32 ones).
-          if (use_tile<T, S>(m, op)) {
-            if constexpr (std::is_same<C, float>::value)
-              launch_tile<TileMom, C, false>(m, p, cf, x, y, nullptr, s);
-            else
-              launch_tile<TileMomQ, C, false>(m, p, cq, x, y, nullptr, s);
-            break;
-          }
-        }
-        launch_patch<MomQK<T, C>, T, S, C, false>(m, p, cq, x, y, nullptr, s);
-        break;
-      }
+      // The persistent kernel evaluates the coefficients in a solve too: faster than reading what
+      // it evaluates, 352 bytes per leaf (momentum solve on 321,112 leaves 16.7 ms against 19.0).
       if constexpr (std::is_same<T, float>::value && std::is_same<S, T>::value) {
         if (use_tile<T, S>(m, op)) {
           launch_tile<TileMom, C, false>(m, p, cf, x, y, nullptr, s);
           break;
         }
+      }
+      // quadrature data of the running momentum solve, when it matches this precision
+      const void* qd = sizeof(T) == sizeof(double) ? m->mq.qd64 : m->mq.qd32;
+      if (m->mq.on && qd) {
+        CoefArgs<C> cq = cf;
+        cq.qd = qd;
+        launch_patch<MomQK<T, C>, T, S, C, false>(m, p, cq, x, y, nullptr, s);
+        break;
       }
       launch_patch<MomK<T, C>, T, S, C, false>(m, p, cf, x, y, nullptr, s);
       break;

@@ -302,11 +302,9 @@ struct PatchBuilder {
     }
     const int nb4 = 4 * nb, n2 = (ns + 1) / 2;
     std::vector<std::array<uint16_t, 16>> ref((size_t)(nb4 + n2));
-    // level and number of leaf k of the patch in the upper bits of entries at, at + 2, at + 4
+    // level of leaf k of the patch in the upper bits of entry at
     auto tag = [&](std::array<uint16_t, 16>& r, int at, int k) {
       r[at] = (uint16_t)(r[at] | (uint32_t)(levels[e0 + k] - low) << 12);
-      r[at + 2] = (uint16_t)(r[at + 2] | (uint32_t)(k & 15) << 12);
-      r[at + 4] = (uint16_t)(r[at + 4] | (uint32_t)(k >> 4) << 12);
     };
     int b = 0, s = 0;
     for (auto& u : units) {

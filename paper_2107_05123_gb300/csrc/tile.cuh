@@ -162,9 +162,9 @@ __device__ __forceinline__ void poisson_cols(const V S[4][2], const V X[4][2], c
 
 // References of a thread's two leaves: byte offsets of their slots in 12 bits of 16. Brick pair
 // (B): node ix + 3 (y + 2 z) of the 3 x 2 x 2 nodes in entry 0..11; others: corner a of the first
-// leaf in entry a, of the second in 8 + a. The upper bits of the even entries hold, for the first
-// leaf (entries 0, 2, 4) and, unless B, the second (8, 10, 12), the level above the patch's
-// lowest and the leaf's number in the patch; entry 6 says whether there is a second leaf.
+// leaf in entry a, of the second in 8 + a. The upper bits of entry 0 and, unless B, entry 8 hold the
+// level of the first leaf and of the second above the patch's lowest; those of entry 6 say whether
+// there is a second leaf.
 template <bool B>
 struct PairRefs {
   const uint32_t* w;
@@ -462,8 +462,7 @@ struct TileCh {
   }
   template <class At>
   static __device__ __forceinline__ void leaf(const float4& c, const PrmT<float>& k, const float* xs,
-                                              const float* fs, const At& at, const float*, int64_t,
-                                              float (&r)[NC][8]) {
+                                              const float* fs, const At& at, float (&r)[NC][8]) {
     constexpr double w = gauss_w<float>(), w3 = w * w * w;
     const Geo<float> g = leaf_geometry(c);
     const float J = g.detJ, *ih = g.ih;
@@ -534,8 +533,7 @@ struct TileMom {
   }
   template <class At>
   static __device__ __forceinline__ void leaf(const float4& c, const PrmT<float>& k, const float* xs,
-                                              const float* fs, const At& at, const float*, int64_t,
-                                              float (&r)[NC][8]) {
+                                              const float* fs, const At& at, float (&r)[NC][8]) {
     const Geo<float> g = leaf_geometry(c);
     VmsFieldsP f;
     {
@@ -569,42 +567,6 @@ struct TileMom {
   }
 };
 
-// The momentum operator from quadrature data (see MomQK), likewise.
-struct TileMomQ {
-  static constexpr int NC = 3;
-  static constexpr int NF = 0;
-  static constexpr bool ONE_PLUS = false, AHEAD = false, DIR = true, ENERGY = false;
-  static constexpr TileForm FORM = TileForm::kLeaf;
-  static constexpr int CTAS = 3;
-  static __device__ __forceinline__ float4 consts(const LevelGeo& g, const PrmT<float>&) {
-    return leaf_consts(g);
-  }
-  // qd: of this leaf
-  template <class At>
-  static __device__ __forceinline__ void leaf(const float4& c, const PrmT<float>&, const float* xs,
-                                              const float*, const At& at, const float* qd, int64_t ne,
-                                              float (&r)[NC][8]) {
-    const Geo<float> g = leaf_geometry(c);
-    float x[NC][8];
-#pragma unroll
-    for (int n = 0; n < NC; ++n)
-#pragma unroll
-      for (int a = 0; a < 8; ++a) x[n][a] = at(xs + n * kPatchSlots, a);
-    momentum_apply_pairs(g, x, r, [&](int q, F2& a0, F2 b[3], F2 bp[3], F2& e, F2 t[3]) {
-      const float* p = qd + (int64_t)(2 * q) * kMomQ * ne;
-      auto pair = [&](int v) { return F2(__ldg(p + v * ne), __ldg(p + (v + kMomQ) * ne)); };
-      a0 = pair(0);
-      e = pair(7);
-#pragma unroll
-      for (int d = 0; d < 3; ++d) {
-        b[d] = pair(1 + d);
-        bp[d] = pair(4 + d);
-        t[d] = pair(8 + d);
-      }
-    });
-  }
-};
-
 // ---------------------------------------------------------------- kernel
 constexpr int kPreSlots = 3;  // regular slots per thread whose values are loaded ahead
 constexpr int kPreHang = 2;   // hanging slots per thread whose parents are loaded ahead
@@ -624,8 +586,7 @@ struct TilePre {
 template <class Op>
 __device__ __forceinline__ void tile_leaves(const PrmT<float>& k, const uint32_t ref[8],
                                             const float4* cst, bool brick, bool any,
-                                            const float* xs, const float* fs, const float* qd,
-                                            int64_t ne, float* yw) {
+                                            const float* xs, const float* fs, float* yw) {
   const PairRefs<true> pr{ref};
   // byte offsets of the corners of both leaves, x = 0 | x = 1 << 16, per x line
   uint32_t o0[4], o1[4];
@@ -638,8 +599,6 @@ __device__ __forceinline__ void tile_leaves(const PrmT<float>& k, const uint32_t
   }
   const bool two = any && (brick || pr.nibble(3) != 0);
   const uint32_t l0 = pr.nibble(0), l1 = brick ? l0 : pr.nibble(4);
-  const uint32_t n0 = pr.nibble(1) | pr.nibble(2) << 4,
-                 n1 = brick ? n0 + 1 : pr.nibble(5) | pr.nibble(6) << 4;  // leaves of the patch
 #pragma unroll 1
   for (int s = 0; s < 2; ++s) {
     const bool active = s ? two : any;
@@ -653,7 +612,7 @@ __device__ __forceinline__ void tile_leaves(const PrmT<float>& k, const uint32_t
       return *reinterpret_cast<const float*>(reinterpret_cast<const char*>(base) + off);
     };
     float r[Op::NC][8];
-    Op::leaf(cst[s ? l1 : l0], k, xs, fs, at, qd + (s ? n1 : n0), ne, r);
+    Op::leaf(cst[s ? l1 : l0], k, xs, fs, at, r);
 #pragma unroll
     for (int a = 0; a < 8; ++a) {
       const uint32_t off = a & 1 ? o[a >> 1] >> 16 : o[a >> 1] & 0xffffu;
@@ -815,8 +774,7 @@ k_apply_tile(MeshDev m, DevParams p, CoefArgs<C> cf, const float* __restrict__ x
     // 2.-3. elements
     float* yw = ys + (tid >> 5) * NC * kPatchSlots;
     if constexpr (Op::FORM == TileForm::kLeaf) {
-      tile_leaves<Op>(k, q.ref, s_cst + (h.w & 0xffffu), tid < nb4, tid < nt, xb, fs,
-                      static_cast<const float*>(cf.qd) + m.patch_elem[t], m.n_elem, yw);
+      tile_leaves<Op>(k, q.ref, s_cst + (h.w & 0xffffu), tid < nb4, tid < nt, xb, fs, yw);
     } else {
       // brick pairs, then the others: a warp that has both takes them one after the other, with all
       // its lanes meeting in between, since a slot can be a corner of leaves of either kind
