@@ -697,70 +697,48 @@ chns_status mg_setup_T(chns_mg* g, int op, cudaStream_t s) {
     chns_status st = level_diag<T>(g, op, l, s);
     if (st != CHNS_OK) return st;
   }
-  // The levels are independent of one another from here on: the coarsest inverse and the power
-  // iterations of the small levels (launch-bound) run on a second stream beside those of the two
-  // finest levels.
+  // Everything on the caller's stream. The coarsest inverse and the small levels' power iterations
+  // beside those of the large levels on a second stream gained 1 to 5 % in Poisson solves (77,932
+  // leaves, FP64 15.7 against 16.5 ms) and lost 4 to 6 % in CH solves (77,932 leaves 17.5 against 16.5
+  // ms, 1,429,744 54.0 against 51.8), and once a process had run kernels on two streams every later
+  // launch of a chain of short kernels took 0.2 us longer.
   const int NS = NL - 1;  // the coarsest level is solved exactly
-  struct Fork {
-    cudaStream_t s, s2;
-    cudaEvent_t e = nullptr;
-    Fork(cudaStream_t a, cudaStream_t b) : s(a), s2(b) {}
-    chns_status order(cudaStream_t from, cudaStream_t to) {
-      if (!e) CHNS_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
-      CHNS_CUDA(cudaEventRecord(e, from));
-      CHNS_CUDA(cudaStreamWaitEvent(to, e, 0));
-      return CHNS_OK;
-    }
-    ~Fork() {  // also after an error: nothing of the second stream outlives the call
-      order(s2, s);
-      if (e) cudaEventDestroy(e);
-    }
-  };
   double* slot = g->slots;
-  {
-    Fork fork(s, g->lv.back().mesh->cap_stream);
-    CHNS_CUDA(cudaMemsetAsync(slot, 0, kMgMaxLevels * sizeof(double), s));
-    chns_status fst = fork.order(s, fork.s2);
-    if (fst != CHNS_OK) return fst;
-    // largest eigenvalue of D^-1 A on level l: power iteration, normalised every kNormEvery steps
-    // (the eigenvalues are of order one) and before the last, whose squared norm goes to the slot
-    constexpr int kNormEvery = 16;
-    auto power = [&](int l, cudaStream_t ps) -> chns_status {
-      MgLevel& L = g->lv[l];
-      T* v = lv_vec<T>(L, 3);
-      T* w = lv_vec<T>(L, 2);
-      note_launch();
-      k_power_start<T><<<grid_for(L.n), kMgThreads, 0, ps>>>(lv_dinv<T>(L, op), v, L.n);
-      const int K = g->prm.power_its;
-      for (int it = 0; it <= K; ++it) {
-        if (it > 0) {
-          chns_status st = level_apply<T>(g, op, l, v, w, ps);
-          if (st != CHNS_OK) return st;
-          note_launch();
-          k_mul<T><<<grid_for(L.n), kMgThreads, 0, ps>>>(lv_dinv<T>(L, op), w, v, L.n);
-        }
-        const bool last = it == K, norm = it == K - 1 || it % kNormEvery == 0;
-        if (!last && !norm) continue;
-        CHNS_CUDA(cudaMemsetAsync(slot + l, 0, sizeof(double), ps));
+  CHNS_CUDA(cudaMemsetAsync(slot, 0, kMgMaxLevels * sizeof(double), s));
+  // largest eigenvalue of D^-1 A on level l: power iteration, normalised every kNormEvery steps (the
+  // eigenvalues are of order one) and before the last, whose squared norm goes to the slot
+  constexpr int kNormEvery = 16;
+  for (int l = 0; l < NS; ++l) {
+    MgLevel& L = g->lv[l];
+    T* v = lv_vec<T>(L, 3);
+    T* w = lv_vec<T>(L, 2);
+    note_launch();
+    k_power_start<T><<<grid_for(L.n), kMgThreads, 0, s>>>(lv_dinv<T>(L, op), v, L.n);
+    const int K = g->prm.power_its;
+    for (int it = 0; it <= K; ++it) {
+      if (it > 0) {
+        chns_status st = level_apply<T>(g, op, l, v, w, s);
+        if (st != CHNS_OK) return st;
         note_launch();
-        k_norm2<T><<<grid_for(L.n), kMgThreads, 0, ps>>>(v, L.n, slot + l);
-        if (last) continue;
-        note_launch();
-        k_normalise<T><<<grid_for(L.n), kMgThreads, 0, ps>>>(v, slot + l, L.n);
+        k_mul<T><<<grid_for(L.n), kMgThreads, 0, s>>>(lv_dinv<T>(L, op), w, v, L.n);
       }
-      return CHNS_OK;
-    };
-    for (int l = 0; l < std::min(NS, 2); ++l) {
-      chns_status st = power(l, s);
-      if (st != CHNS_OK) return st;
+      const bool last = it == K, norm = it == K - 1 || it % kNormEvery == 0;
+      if (!last && !norm) continue;
+      CHNS_CUDA(cudaMemsetAsync(slot + l, 0, sizeof(double), s));
+      note_launch();
+      k_norm2<T><<<grid_for(L.n), kMgThreads, 0, s>>>(v, L.n, slot + l);
+      if (last) continue;
+      note_launch();
+      k_normalise<T><<<grid_for(L.n), kMgThreads, 0, s>>>(v, slot + l, L.n);
     }
-    cudaStream_t cs = fork.s2;
+  }
+  {
     // coarsest: dense inverse in FP64 (Poisson: of A + 1 1^T / n, the mean-zero solution)
     MgLevel& C = g->lv.back();
     const int n = (int)C.n;
     // the FP32 setup works in its own FP64 matrix, so that the FP64 inverse stays valid
     double* Aw = sizeof(T) == sizeof(double) ? O.cinv64 : g->cwork64;
-    CHNS_CUDA(cudaMemsetAsync(Aw, 0, (size_t)n * n * sizeof(double), cs));
+    CHNS_CUDA(cudaMemsetAsync(Aw, 0, (size_t)n * n * sizeof(double), s));
     DevParams p = make_dev_params(g->phys);
     CoefArgs<double> cf{};
     cf.phi_shift = 0.0f;
@@ -773,18 +751,18 @@ chns_status mg_setup_T(chns_mg* g, int op, cudaStream_t s) {
         // FP64 copy of the FP32 coefficients in the coarsest level's FP64 apply-output vector
         double* tmp = C.v64[2];
         note_launch();
-        k_convert<T, double><<<grid_for(n), kMgThreads, 0, cs>>>(level_phi<T>(g, NL - 1), tmp, n);
+        k_convert<T, double><<<grid_for(n), kMgThreads, 0, s>>>(level_phi<T>(g, NL - 1), tmp, n);
         phic = tmp;
       }
       cf.phi = phic;
       note_launch();
-      k_dense_assemble<PoissonK<double, double>><<<nb, 128, 0, cs>>>(C.mesh->d, p, cf, Aw, n);
+      k_dense_assemble<PoissonK<double, double>><<<nb, 128, 0, s>>>(C.mesh->d, p, cf, Aw, n);
     } else {
       p.d.sa = O.sa;
       p.d.sb = O.sb;
       cf.phi = C.v64[2];  // gathered, unused
       note_launch();
-      k_dense_assemble<ShiftK<double, double>><<<nb, 128, 0, cs>>>(C.mesh->d, p, cf, Aw, n);
+      k_dense_assemble<ShiftK<double, double>><<<nb, 128, 0, s>>>(C.mesh->d, p, cf, Aw, n);
     }
     const bool in_smem = n <= kGjSmem;
     const size_t smem = in_smem ? (size_t)n * n * sizeof(double) : 0;
@@ -792,15 +770,11 @@ chns_status mg_setup_T(chns_mg* g, int op, cudaStream_t s) {
       CHNS_CUDA(cudaFuncSetAttribute(k_gauss_jordan, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      kGjSmem * kGjSmem * (int)sizeof(double)));
     note_launch();
-    k_gauss_jordan<<<1, 1024, smem, cs>>>(Aw, n, op == kMgPoisson ? 1.0 / n : 0.0, in_smem);
+    k_gauss_jordan<<<1, 1024, smem, s>>>(Aw, n, op == kMgPoisson ? 1.0 / n : 0.0, in_smem);
     if (sizeof(T) == sizeof(float)) {
       note_launch();
-      k_convert<double, float><<<grid_for((int64_t)n * n), kMgThreads, 0, cs>>>(
+      k_convert<double, float><<<grid_for((int64_t)n * n), kMgThreads, 0, s>>>(
           Aw, O.cinv32, (int64_t)n * n);
-    }
-    for (int l = 2; l < NS; ++l) {
-      chns_status st = power(l, cs);
-      if (st != CHNS_OK) return st;
     }
   }
   if (NS > 0)
