@@ -292,6 +292,14 @@ static bool tile_writes_rows(const chns_mesh* m, chns_operator op) {
   return (op == CHNS_OP_MASS || op == CHNS_OP_MOMENTUM) && use_tile<float, float>(m, op);
 }
 
+// The quadrature data of the running momentum solve in precision T, if it has any.
+template <class T>
+static const void* momentum_qdata(const chns_mesh* m) {
+  if (!m->mq.on) return nullptr;
+  if (sizeof(T) == sizeof(double)) return m->mq.qd64;
+  return m->mq.has32 ? m->mq.qd32 : nullptr;
+}
+
 // Reference (corner a, slot k) -> node reference with Dirichlet bit and its weight, or -1.
 __device__ __forceinline__ int corner_ref(const MeshDev& m, int v, int k, double& w) {
   int j = v & kIdxMask;
@@ -459,9 +467,8 @@ static void launch_apply(const chns_mesh* m, chns_operator op, const DevParams& 
           break;
         }
       }
-      // quadrature data of the running momentum solve, when it matches this precision
-      const void* qd = sizeof(T) == sizeof(double) ? m->mq.qd64 : m->mq.qd32;
-      if (m->mq.on && qd) {
+      // quadrature data of the running momentum solve, when there are any in this precision
+      if (const void* qd = momentum_qdata<T>(m)) {
         CoefArgs<C> cq = cf;
         cq.qd = qd;
         launch_patch<MomQK<T, C>, T, S, C, false>(m, p, cq, x, y, nullptr, s);
@@ -482,8 +489,10 @@ static void launch_apply_df(const chns_mesh* m, chns_operator op, const DevParam
     launch_patch<MassK<DF, double>, DF, double, double, false>(m, p, cf, x, y, nullptr, s);
 }
 
-// Quadrature data of the momentum operator for the coefficients coef (FP64 and, when coef32 is
-// given, FP32), used by every momentum apply until momentum_qdata_off.
+// Quadrature data of the momentum operator for the coefficients coef, used by every momentum apply and
+// diagonal of that precision until momentum_qdata_off: FP64 and, when coef32 is given and the FP32
+// applies take the CTA-per-patch kernel, FP32. The persistent kernel evaluates its coefficients, and
+// so does the diagonal then: 6.0 ms on 6.9e6 leaves, 21 from the data, 352 bytes per leaf.
 chns_status momentum_qdata_on(const chns_mesh* m, const chns_params* prm, const chns_coef* coef64,
                               const chns_coef* coef32, cudaStream_t s) {
   chns_status st = check_coef(CHNS_OP_MOMENTUM, coef64);
@@ -491,20 +500,21 @@ chns_status momentum_qdata_on(const chns_mesh* m, const chns_params* prm, const 
   const int64_t E = m->d.n_elem;
   const size_t nv = (size_t)8 * kMomQ * E;
   if (!m->mq.qd64) CHNS_CUDA(cudaMalloc(&m->mq.qd64, nv * sizeof(double)));
-  if (coef32 && !m->mq.qd32) CHNS_CUDA(cudaMalloc(&m->mq.qd32, nv * sizeof(float)));
+  const bool with32 = coef32 && !use_tile<float, float>(m, CHNS_OP_MOMENTUM);
+  if (with32 && !m->mq.qd32) CHNS_CUDA(cudaMalloc(&m->mq.qd32, nv * sizeof(float)));
   const DevParams p = make_dev_params(*prm);
   const unsigned nb = (unsigned)((E + 127) / 128);
   note_launch();
   k_mom_qdata<double, double><<<nb, 128, 0, s>>>(m->d, p, coef_args<double>(coef64),
                                                  static_cast<double*>(m->mq.qd64));
-  if (coef32) {
+  if (with32) {
     note_launch();
     k_mom_qdata<float, float><<<nb, 128, 0, s>>>(m->d, p, coef_args<float>(coef32),
                                                  static_cast<float*>(m->mq.qd32));
   }
   CHNS_CUDA(cudaGetLastError());
   m->mq.on = true;
-  m->mq.has32 = coef32 != nullptr;
+  m->mq.has32 = with32;
   return CHNS_OK;
 }
 
@@ -530,10 +540,9 @@ static void launch_diag(const chns_mesh* m, chns_operator op, const DevParams& p
       break;
     case CHNS_OP_MOMENTUM: {
       note_launch();
-      // from the quadrature data of the running momentum solve when it matches this precision
-      // (the operator the solve applies; the direct form re-evaluates tau_m per point)
-      const void* qd = sizeof(T) == sizeof(double) ? m->mq.qd64 : m->mq.qd32;
-      if (m->mq.on && qd) {
+      // from the quadrature data of the running momentum solve when there are any in this precision
+      // (the operator the solve applies)
+      if (const void* qd = momentum_qdata<T>(m)) {
         CoefArgs<C> cq = cf;
         cq.qd = qd;
         k_diag<MomQK<T, C>, T, S, C><<<nb, kApplyThreads, 0, s>>>(m->d, p, cq, d);

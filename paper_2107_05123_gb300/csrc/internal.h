@@ -202,7 +202,8 @@ chns_status apply_poisson_cg(const chns_mesh* m, const chns_params* prm, const c
                              chns_precision prec, double* S_cg, int par, cudaStream_t s,
                              bool fcg = false);
 // Precompute the momentum operator's quadrature data for coefficients that stay fixed over the
-// applies that follow (a Krylov solve); momentum_qdata_off returns to on-the-fly evaluation.
+// applies that follow (a Krylov solve), in the precisions whose kernels read them;
+// momentum_qdata_off returns to on-the-fly evaluation.
 chns_status momentum_qdata_on(const chns_mesh* m, const chns_params* prm, const chns_coef* coef64,
                               const chns_coef* coef32, cudaStream_t s);
 void momentum_qdata_off(const chns_mesh* m);
