@@ -34,15 +34,19 @@ __device__ __forceinline__ void reduce_finalize(A (&v)[NV], double* __restrict__
   block_reduce_finalize<NV, kVecThreads>(v, part, kRedSlots, counter, out);
 }
 
-// Vector kernels that read several arrays and write others: kBatch elements per thread and round,
-// all of a round's loads before its first store (the compiler keeps the order of loads and stores
-// it cannot tell apart, which left one element's round trip to memory exposed per iteration).
-constexpr int kBatch = 4;
-#define BATCH_LOOP(i0, n)                                                    \
+// Vector kernels that read several arrays and write others: B elements per thread and round, all of a
+// round's loads before its first store (the compiler keeps the order of loads and stores it cannot
+// tell apart, which left one element's round trip to memory exposed per iteration). Two are best in
+// FP32: with four a thread's predicated loads and registers cost more than they hide on all but the
+// longest vectors, with one the longest suffer. Iterations with B = 1 / 2 / 4: Jacobi-CG on 129,409
+// nodes 7.9 / 7.7 / 10.3 ms a solve, 1,216,473 nodes 53.6 / 46.0 / 53.7 us each; Chebyshev there 151 /
+// 139 / 143 us; multigrid solve on 6.0e6 nodes 60.4 / 54.7 / 54.9 ms. In FP64 CG one is enough (Jacobi-CG
+// for the mass operator on 1,216,473 nodes 54.2 / 54.9 / 54.3 ms).
+#define BATCH_LOOP(B, i0, n)                                                 \
   for (int64_t i0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i0 < (n); \
-       i0 += (int64_t)kBatch * gridDim.x * blockDim.x)
-#define BATCH(u, i, i0, n)                                                              \
-  _Pragma("unroll") for (int u = 0; u < kBatch; ++u)                                    \
+       i0 += (int64_t)(B) * gridDim.x * blockDim.x)
+#define BATCH(B, u, i, i0, n)                                                           \
+  _Pragma("unroll") for (int u = 0; u < (B); ++u)                                       \
     if (const int64_t i = i0 + (int64_t)u * gridDim.x * blockDim.x; i < (n))
 
 #define GRID_LOOP(i, n)                                                     \
@@ -176,18 +180,19 @@ __global__ void __launch_bounds__(kVecThreads)
 k_cg_update(T* __restrict__ x, T* __restrict__ r, T* __restrict__ z, const T* __restrict__ p,
             T* __restrict__ q, const T* __restrict__ dinv, int64_t n, double* __restrict__ S,
             bool zero_q, int par) {
+  constexpr int B = sizeof(T) == 4 ? 2 : 1;
   const T a = cg_ratio<T>(S, kCgRz0 + par, kCgPq0 + par, true);
   typename Acc<T>::type v0 = Acc<T>::zero(), v1 = Acc<T>::zero();
-  BATCH_LOOP(i0, n) {
-    T xv[kBatch], pv[kBatch], rv[kBatch], qv[kBatch], dv[kBatch];
-    BATCH(u, i, i0, n) {
+  BATCH_LOOP(B, i0, n) {
+    T xv[B], pv[B], rv[B], qv[B], dv[B];
+    BATCH(B, u, i, i0, n) {
       xv[u] = x[i];
       pv[u] = p[i];
       rv[u] = r[i];
       qv[u] = q[i];
       dv[u] = dinv ? dinv[i] : T(1);
     }
-    BATCH(u, i, i0, n) {
+    BATCH(B, u, i, i0, n) {
       x[i] = xv[u] + a * pv[u];
       const T ri = rv[u] - a * qv[u];
       if (zero_q) q[i] = T(0);
@@ -243,17 +248,18 @@ template <class T>
 __global__ void __launch_bounds__(kVecThreads)
 k_fcg_update(T* __restrict__ x, T* __restrict__ r, const T* __restrict__ p,
              const T* __restrict__ q, int64_t n, double* __restrict__ S, int par) {
+  constexpr int B = 2;
   const T a = cg_ratio<T>(S, kFcgRz0 + par, kCgPq0 + par, true);
   typename Acc<T>::type v0 = Acc<T>::zero();
-  BATCH_LOOP(i0, n) {
-    T xv[kBatch], pv[kBatch], rv[kBatch], qv[kBatch];
-    BATCH(u, i, i0, n) {
+  BATCH_LOOP(B, i0, n) {
+    T xv[B], pv[B], rv[B], qv[B];
+    BATCH(B, u, i, i0, n) {
       xv[u] = x[i];
       pv[u] = p[i];
       rv[u] = r[i];
       qv[u] = q[i];
     }
-    BATCH(u, i, i0, n) {
+    BATCH(B, u, i, i0, n) {
       x[i] = xv[u] + a * pv[u];
       const T ri = rv[u] - a * qv[u];
       r[i] = ri;
@@ -279,15 +285,16 @@ template <class T>
 __global__ void __launch_bounds__(kVecThreads)
 k_fcg_dots(const T* __restrict__ z, T* __restrict__ q, const T* __restrict__ r, int64_t n,
            double* __restrict__ S, int par) {
+  constexpr int B = 2;
   typename Acc<T>::type v0 = Acc<T>::zero(), v1 = Acc<T>::zero();
-  BATCH_LOOP(i0, n) {
-    T zv[kBatch], qv[kBatch], rv[kBatch];
-    BATCH(u, i, i0, n) {
+  BATCH_LOOP(B, i0, n) {
+    T zv[B], qv[B], rv[B];
+    BATCH(B, u, i, i0, n) {
       zv[u] = z[i];
       qv[u] = q[i];
       rv[u] = r[i];
     }
-    BATCH(u, i, i0, n) {
+    BATCH(B, u, i, i0, n) {
       q[i] = T(0);
       Acc<T>::fma(v0, zv[u], qv[u]);
       Acc<T>::fma(v1, zv[u], rv[u]);

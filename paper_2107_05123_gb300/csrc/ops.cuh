@@ -9,9 +9,9 @@
 // constants, Kronecker products for the constant-coefficient terms, physical scalings on the 12
 // compact gradient values instead of at 8 points, one reciprocal and one reciprocal square root
 // per point by a third-order step from the hardware estimate, comparisons in integers. FP64 applies
-// of all four operators on 156,640 leaves: 1,562 -> 918 us; the four FP64 right-hand sides and
-// residuals on 314,672 leaves 4.82 -> 3.73 ms; FP32 momentum there 76.8 -> 55.9 us in
-// the CTA-per-patch kernel (41.1 us as TileMom).
+// of all four operators on 156,640 leaves: 1,562 -> 923 us; the four FP64 right-hand sides and
+// residuals on 314,672 leaves 4.82 -> 3.83 ms; FP32 momentum there 76.8 -> 55 us in
+// the CTA-per-patch kernel (41.3 us as TileMom).
 #pragma once
 
 #include <type_traits>

@@ -24,9 +24,9 @@
 // values, parents and references of k + 1, all in registers, so that no phase waits for a load
 // it has just issued.
 //
-// What bounds it: latency and issue together (62 % of the issue slots, short scoreboard and wait
-// stalls), on large meshes also the index records (21 bytes per leaf of 35). Measured against one
-// thread per leaf with shared-memory float atomics (a compare-and-swap loop on this part, 5.3 cycles
+// What bounds it: latency and issue together (Poisson on 1,429,744 leaves: 59 % of the issue slots,
+// barrier and short scoreboard stalls), on large meshes also the index records (21 bytes per leaf of
+// 35). Measured against one thread per leaf with shared-memory float atomics (a compare-and-swap loop on this part, 5.3 cycles
 // per warp operation against 2.1 for the read-add-write and 26 against 9.6 in latency): Poisson
 // on 6.9e6 leaves 185 -> 147 us, mass (bfloat16 coefficients) on 3.1e5 32.7 -> 28.0 us with the
 // identity rows' kernel gone. Also measured, slower (Poisson, 6.9e6 leaves): one warp per patch
