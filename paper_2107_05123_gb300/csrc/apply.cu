@@ -269,8 +269,8 @@ static void launch_tile(const chns_mesh* m, const DevParams& p, const CoefArgs<C
 // FP32 vectors take the two-leaves-per-thread kernel from kTilePatchesPerSm patches per SM on: its
 // CTAs then have patches to load ahead, while on smaller meshes, where one patch's latency is the
 // whole time, the CTA-per-patch kernel with one leaf per thread is as fast or faster (measured in
-// a CUDA graph, per-patch / this: Poisson on 19,608 leaves 5.8 / 6.5 us, 77,932 6.7 / 7.1, 156,640
-// 8.1 / 8.2, 314,672 (8.2 patches per SM) 12.9 / 11.8, 635,328 17.7 / 15.6, 1,429,744 38.7 / 32.9; mass
+// a CUDA graph, per-patch / this: Poisson on 19,608 leaves 5.6 / 6.5 us, 77,932 6.7 / 7.1, 156,640
+// 7.8 / 8.2, 314,672 (8.2 patches per SM) 12.5 / 11.9, 635,328 18.0 / 15.6, 1,429,744 39.9 / 33.0; mass
 // on 156,640 14.8 / 14.7, 314,672 24.6 / 23.0, 635,328 33.4 / 35.0, 756,064 40.6 / 40.5, 1,429,744
 // 80.5 / 74.9).
 constexpr int kTilePatchesPerSm = 8;

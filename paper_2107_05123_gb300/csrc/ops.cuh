@@ -46,9 +46,10 @@ __device__ __forceinline__ void gather_phi(const MeshDev& m, const int idx[8],
 template <class T, class C>
 struct PoissonK {
   static constexpr bool QDATA = false;
-  // CTAs of the patch apply resident per SM that the register allocation must allow (FP32: 6,
-  // i.e. at most 42 registers; FP64: 3)
-  static constexpr int MIN_CTAS = sizeof(T) == 4 ? 6 : 3;
+  // CTAs of the patch apply resident per SM that the register allocation must allow (FP32: 5, i.e. at
+  // most 51 registers; FP64: 3). Meshes of up to 8 patches per SM take this kernel in FP32: at 6 CTAs
+  // and 40 registers it spills, 6.9 us on 77,932 leaves and 8.1 on 156,640 against 6.7 and 7.8.
+  static constexpr int MIN_CTAS = sizeof(T) == 4 ? 5 : 3;
   static constexpr int NC = 1;
   static constexpr bool DIR = false;
   static constexpr bool DIAG_PER_COMP = false;
