@@ -48,10 +48,10 @@ UNIT = "DOFs/s"
 WORKLOAD = "rayleigh_taylor_levels6-10"
 # DRAM bytes of one launch of the roofline kernel on the headline mesh (ncu
 # dram__bytes_read.sum + dram__bytes_write.sum, summarised under profiles/); --traffic overrides
-APPLY_DRAM_BYTES = 265.2e6  # mean of two launches (ncu capture summarised under profiles/)
+APPLY_DRAM_BYTES = 230.5e6  # mean of two launches (ncu capture summarised under profiles/)
 # FP64 flops per element of the standalone FP64 applies (2 DFMA + DADD + DMUL thread
 # instructions per leaf, one ncu capture on the levels 6-9 Rayleigh-Taylor mesh, profiles/)
-FP64_FLOPS_PER_ELEM = {"poisson": 423.1, "mass": 517.1, "ch": 1085.0, "momentum": 4582.5}
+FP64_FLOPS_PER_ELEM = {"poisson": 325.1, "mass": 434.0, "ch": 759.9, "momentum": 2357.4}
 # the reference arm's bounded sample of the headline workload: the same interface, box and
 # physics on levels 5-8
 SAMPLE_LEVELS = (5, 8)
